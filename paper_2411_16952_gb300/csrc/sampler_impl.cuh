@@ -983,69 +983,212 @@ static __device__ double poisson_tail_d(double lambda, int k) {
 constexpr int kMaxCopies = (1 << 24) - 1;  // copies fit the record's 24-bit field
 
 // ---- FP64 decision of the guard-band proposals ---------------------------
+// A warp takes up to 32 queued proposals.  The K modes of a proposal and its
+// triads are spread over a segment of kLanes lanes (32 / kLanes proposals at
+// a time), their sums meet in the segment by shuffles, and lane q keeps those
+// of proposal q; the scalar part of the decision (1/|x|, the logarithms, the
+// SIR copy number) then runs once for the whole batch, a proposal per lane.
+//
+// What bounds it: an FP64 instruction of a warp holds its scheduler for 64
+// cycles (measured, dependent or not, whatever the number of active lanes).
+// One thread per proposal made K log/sincos pairs and 2 K^2 FMAs in series,
+// and a run waits for the one queued proposal as long as for thousands: 88,
+// 207 and 600 us per run at 16, 32 and 64 modes.  Spread over the lanes the
+// same FP64 work is about 400, 400 and 700 warp instructions: a run of 2^16
+// proposals at 16 modes went from 166 to 94 us (static call), one of 2^25 at
+// 64 modes from 7.04 to 6.40 ms, of 8 x 2^22 at 32 modes from 4.03 to 3.82 ms.
+// With a full queue both forms need about the same number of FP64 warp
+// instructions per proposal, so there is one form only.
+template <int KMAX>
+struct RefineShape {
+    static constexpr int kLanes = KMAX < 8 ? 8 : KMAX < 32 ? KMAX : 32;  // lanes of one proposal
+    static constexpr int kGroup = 32 / kLanes;                          // proposals at a time
+    static constexpr int kModes = KMAX / kLanes > 1 ? KMAX / kLanes : 1;  // modes of one lane
+    static constexpr int kBatch = 32;
+    static constexpr int kWarps = 4;
+    static constexpr size_t kSmem = sizeof(double2) * kWarps * kBatch * KMAX;
+};
+
+// Sums over a segment's lanes, the same values in every lane of it.
+template <int LANES>
+__device__ __forceinline__ double seg_sum(double v) {
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 template <int KMAX, bool UNIF>
 __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t k1) {
+    using RS = RefineShape<KMAX>;
+    constexpr int LANES = RS::kLanes, GROUP = RS::kGroup, MODES = RS::kModes;
+    extern __shared__ __align__(16) unsigned char s_refine[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane / LANES, l = lane % LANES;
+    double2 *slab = reinterpret_cast<double2 *>(s_refine) + (size_t)warp * RS::kBatch * KMAX;
     const uint32_t n = min(*(volatile uint32_t *)&B.counters[1], B.refine_cap);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const RefineItem it = B.refine[i];
+    // batches of consecutive items, first to distinct CTAs, then to the warps
+    // of a CTA (one per scheduler), as small as the warps allow
+    const uint32_t nw = gridDim.x * RS::kWarps;
+    uint32_t batch = (n + nw - 1) / nw;
+    batch = min((batch + GROUP - 1) / GROUP * GROUP, (uint32_t)RS::kBatch);
+    for (uint32_t first = ((uint32_t)warp * gridDim.x + blockIdx.x) * batch; first < n; first += nw * batch) {
+        const uint32_t cnt = min(batch, n - first);
+        double nrm2 = 1.0, Sraw = 0.0, zz = 1.0, u0raw = 0.0, T = 0.0;  // of item first + lane
+        __syncwarp();  // the slab's readers of the previous batch are done
+#pragma unroll 1
+        for (uint32_t g0 = 0; g0 < cnt; g0 += GROUP) {
+            const uint32_t q = min(g0 + (uint32_t)sub, cnt - 1);  // (an idle segment repeats the last item)
+            const RefineItem it = B.refine[first + q];
+            const PointConst *P = B.pts + it.point;
+            const int K = P->K;
+            const uint32_t lo = (uint32_t)it.idx, hi = (uint32_t)(it.idx >> 32), pid = P->point_id;
+            double2 *sx = slab + (size_t)(g0 + (uint32_t)sub) * KMAX;
+            double an = 0.0, aS = 0.0, az = 0.0, au = 0.0;
+#pragma unroll 1
+            for (int i = 0; i < MODES; ++i) {
+                const int m = MODES * l + i;
+                double2 v = make_double2(0.0, 0.0);
+                if (m < K) {
+                    const uint4 w = philox4x32_10(make_uint4((uint32_t)(m / 2), lo, hi, pid), k0, k1);
+                    const int h = m & 1;
+                    const double u1 = u01d_ext(h ? w.z : w.x, 2u * (uint32_t)m, lo, hi, pid, k0, k1);
+                    const double u2 = u01d(h ? w.w : w.y);
+                    const double rho = -2.0 * log(u1);
+                    const double rad = sqrt(rho);
+                    double sn, cs;
+                    sincospi(2.0 * u2, &sn, &cs);
+                    const double s = UNIF ? 1.0 : P->sigma_d[m];
+                    v.x = s * rad * cs;
+                    v.y = s * rad * sn;
+                    const double sk = v.x * v.x + v.y * v.y;
+                    an += sk;
+                    aS += (double)((m + 1) * (m + 1)) * sk;
+                    az += rho;
+                    au += v.x;
+                }
+                if (m < KMAX) sx[m] = v;
+            }
+            __syncwarp();
+            // T = sum over k <= l, k + l <= KMAX of w Re(v_k v_l conj(v_{k+l})),
+            // w = 2 for k < l, else 1.  Row k holds the KMAX - 2k + 1 values
+            // l = k..KMAX-k; rows k and KMAX/2 + 1 - k together hold KMAX, so
+            // the KMAX^2/4 triads are numbered by (row pair, place in it).
+            double at = 0.0;
+#pragma unroll 2
+            for (int e = l; e < KMAX * KMAX / 4; e += LANES) {
+                const int rp = e / KMAX, c = e % KMAX, len = KMAX - 2 * rp - 1;
+                const int kk = c < len ? rp + 1 : KMAX / 2 - rp;
+                const int ll = c < len ? kk + c : kk + (c - len);
+                const double2 a = sx[kk - 1], b = sx[ll - 1], v = sx[kk + ll - 1];
+                const double A = fma(a.x, b.x, -(a.y * b.y)), Bv = fma(a.x, b.y, a.y * b.x);
+                at = fma(kk < ll ? 2.0 : 1.0, fma(v.x, A, v.y * Bv), at);
+            }
+            an = seg_sum<LANES>(an);
+            aS = seg_sum<LANES>(aS);
+            az = seg_sum<LANES>(az);
+            au = seg_sum<LANES>(au);
+            at = seg_sum<LANES>(at);
+            // lane g0 + s takes the sums of segment s
+            const int src = ((lane - (int)g0) & (GROUP - 1)) * LANES;
+            const double on = __shfl_sync(0xffffffffu, an, src), oS = __shfl_sync(0xffffffffu, aS, src),
+                         oz = __shfl_sync(0xffffffffu, az, src), ou = __shfl_sync(0xffffffffu, au, src),
+                         ot = __shfl_sync(0xffffffffu, at, src);
+            if (lane >= (int)g0 && lane < (int)g0 + GROUP) {
+                nrm2 = on;
+                Sraw = oS;
+                zz = oz;
+                u0raw = ou;
+                T = ot;
+            }
+        }
+        // the decision of item first + lane (the formulas of eval64)
+        const bool valid = (uint32_t)lane < cnt;
+        const RefineItem it = B.refine[first + min((uint32_t)lane, cnt - 1)];
         const PointConst *P = B.pts + it.point;
         StatBlock *st = B.stats + it.point;
-        Out64 o;
-        float xh[2 * KMAX];
-        eval64<KMAX, UNIF>(P, it.idx, k0, k1, &o, xh);
-        atomicAdd(&st->n_refined, 1ull);
-        atomicMax(&st->maxd_key, (unsigned long long)fkey((float)o.delta));
-        unsigned long long copies = 1;
-        if (B.sir) {
-            // SIR: n = #{k >= 1 : U < P(N >= k)}, N ~ Poisson(c exp(delta))
-            const double lam = P->sir_c * exp(o.delta);
-            int n = 0;
-            double tk = poisson_tail_d(lam, 1);
-            while (n < kMaxCopies && o.u < tk) {
-                ++n;
-                tk = poisson_tail_d(lam, n + 1);
+        const int K = P->K;
+        const double inv = 1.0 / sqrt(nrm2);
+        unsigned long long copies = 0;
+        bool near = false;
+        double S = 0.0, Tn = 0.0, delta = 0.0;
+        if (valid) {
+            const uint32_t lo = (uint32_t)it.idx, hi = (uint32_t)(it.idx >> 32), pid = P->point_id;
+            const double inv2 = inv * inv;
+            S = Sraw * inv2;
+            Tn = T * inv2 * inv;
+            delta = P->cS_d * S + P->cH_d * Tn;
+            if (!UNIF) delta += P->cQ_d * log(zz * inv2);
+            delta -= P->logM;
+            const uint32_t wa = accept_word(lo, hi, pid, K, k0, k1);
+            const double u = u01d_ext(wa, 4u * (uint32_t)((K + 1) / 2), lo, hi, pid, k0, k1);
+            const double lnU = log(u);
+            near = fabs(lnU - delta) < 1e-6;
+            atomicAdd(&st->n_refined, 1ull);
+            atomicMax(&st->maxd_key, (unsigned long long)fkey((float)delta));
+            if (B.sir) {
+                // SIR: n = #{k >= 1 : U < P(N >= k)}, N ~ Poisson(c exp(delta))
+                const double lam = P->sir_c * exp(delta);
+                int nc = 0;
+                double tk = poisson_tail_d(lam, 1);
+                while (nc < kMaxCopies && u < tk) {
+                    ++nc;
+                    tk = poisson_tail_d(lam, nc + 1);
+                }
+                // near: U within 1e-6 (in log) of the tail value that decided n
+                const double tn = nc > 0 ? poisson_tail_d(lam, nc) : 1.0;
+                near = fabs(lnU - log(tk)) < 1e-6 || (nc > 0 && fabs(lnU - log(tn)) < 1e-6);
+                if (nc > 0) atomicAdd(&st->n_kept, 1ull);
+                copies = (unsigned long long)nc;
+            } else {
+                if (delta > 0.0) atomicAdd(&st->n_viol, 1ull);
+                copies = lnU < delta ? 1ull : 0ull;
             }
-            // near: U within 1e-6 (in log) of the tail value that decided n
-            const double tn = n > 0 ? poisson_tail_d(lam, n) : 1.0;
-            const bool near = fabs(o.lnU - log(tk)) < 1e-6 || (n > 0 && fabs(o.lnU - log(tn)) < 1e-6);
-            o.near = near;
             if (near) atomicAdd(&st->n_near, 1ull);
-            if (n == 0) continue;
-            atomicAdd(&st->n_kept, 1ull);
-            copies = (unsigned long long)n;
-        } else {
-            if (o.near) atomicAdd(&st->n_near, 1ull);
-            if (o.delta > 0.0) atomicAdd(&st->n_viol, 1ull);
-            if (!o.accept) continue;
         }
-        atomicAdd(&st->n_acc, copies);
-        const float u0 = o.u0;
-        atomicAdd(&st->hist[hist_bin(u0, __ldg(&P->hist_a), __ldg(&P->hist_b))], copies);
-        atomicAdd(&st->exc[exc_bin(u0, __ldg(&P->exc_a))], copies);
-        const float u2 = u0 * u0;
-        atomicAdd(&st->q[0], copies * (unsigned long long)__float2ll_rn(u0 * kQ1));
-        atomicAdd(&st->q[1], copies * (unsigned long long)__float2ll_rn(u2 * kQ2));
-        atomicAdd(&st->q[2], copies * (unsigned long long)__float2ll_rn(u2 * u0 * kQ3));
-        atomicAdd(&st->q[3], copies * (unsigned long long)__float2ll_rn(u2 * u2 * kQ4));
-        for (int m = 0; m < P->K; ++m)
-            atomicAdd(&st->spec[m], copies * (unsigned long long)__float2ull_rn(
-                                                 fmaf(xh[m], xh[m], xh[P->K + m] * xh[P->K + m]) * kSpecScale));
-        const unsigned long long slot = atomicAdd(B.ring_count, 1ull);
-        if (slot < B.ring_cap) {
-            const int K = P->K;
-            unsigned char *rec = B.ring + slot * B.rec_bytes;
-            *reinterpret_cast<unsigned long long *>(rec) = it.idx;
-            uint32_t *h = reinterpret_cast<uint32_t *>(rec + 8);
-            h[0] = it.point;
-            h[1] = 1u | (o.near ? 2u : 0u) | (B.sir ? (uint32_t)copies << 8 : 0u);
-            float *f = reinterpret_cast<float *>(rec + 16);
-            f[0] = o.H2;
-            f[1] = o.H3;
-            f[2] = o.u0;
-            f[3] = (float)o.delta;
-            for (int m = 0; m < 2 * K; ++m) f[4 + m] = xh[m];
-        } else {
-            atomicAdd(&st->n_dropped, 1ull);
+        // outputs: the lane's scalars, then the states, one proposal at a time
+        unsigned mk = __ballot_sync(0xffffffffu, copies > 0);
+        if (!mk) continue;
+        unsigned long long slot0 = 0;
+        if (lane == 0) slot0 = atomicAdd(B.ring_count, (unsigned long long)__popc(mk));
+        slot0 = __shfl_sync(0xffffffffu, slot0, 0);
+        unsigned char *rec = nullptr;
+        if (copies > 0) {
+            const float u0 = (float)((double)P->u0s * u0raw * inv), u2 = u0 * u0;
+            atomicAdd(&st->n_acc, copies);
+            atomicAdd(&st->hist[hist_bin(u0, __ldg(&P->hist_a), __ldg(&P->hist_b))], copies);
+            atomicAdd(&st->exc[exc_bin(u0, __ldg(&P->exc_a))], copies);
+            atomicAdd(&st->q[0], copies * (unsigned long long)__float2ll_rn(u0 * kQ1));
+            atomicAdd(&st->q[1], copies * (unsigned long long)__float2ll_rn(u2 * kQ2));
+            atomicAdd(&st->q[2], copies * (unsigned long long)__float2ll_rn(u2 * u0 * kQ3));
+            atomicAdd(&st->q[3], copies * (unsigned long long)__float2ll_rn(u2 * u2 * kQ4));
+            const unsigned long long slot = slot0 + __popc(mk & ((1u << lane) - 1u));
+            if (slot < B.ring_cap) {
+                rec = B.ring + slot * B.rec_bytes;
+                write_header(rec, it.idx, it.point, 1u | (near ? 2u : 0u) | (B.sir ? (uint32_t)copies << 8 : 0u),
+                             (float)((double)P->E0 * S), (float)((double)P->h3s * Tn), u0, (float)delta);
+            } else {
+                atomicAdd(&st->n_dropped, 1ull);
+            }
+        }
+        while (mk) {
+            const int q = __ffs(mk) - 1;
+            mk &= mk - 1;
+            const double qinv = __shfl_sync(0xffffffffu, inv, q);
+            const unsigned long long qc = __shfl_sync(0xffffffffu, copies, q);
+            const uint32_t qp = __shfl_sync(0xffffffffu, it.point, q);
+            const int qK = __shfl_sync(0xffffffffu, K, q);
+            float *xh =
+                reinterpret_cast<float *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(rec), q));
+            const double2 *sx = slab + (size_t)q * KMAX;
+            for (int m = lane; m < qK; m += 32) {
+                const double2 v = sx[m];
+                const float x = (float)(v.x * qinv), y = (float)(v.y * qinv);
+                atomicAdd(&B.stats[qp].spec[m], qc * (unsigned long long)__float2ull_rn(fmaf(x, x, y * y) * kSpecScale));
+                if (xh) {
+                    xh[8 + m] = x;
+                    xh[8 + qK + m] = y;
+                }
+            }
         }
     }
 }
@@ -1136,6 +1279,7 @@ void fill_triad_kernels_xfer(TriadKernels *t) {
     t->sir[1] = (const void *)k_sample_triad<KMAX, true, 256, 1, true, false>;
     t->refine[0] = (const void *)k_refine<KMAX, false>;
     t->refine[1] = (const void *)k_refine<KMAX, true>;
+    t->refine_smem = (int)RefineShape<KMAX>::kSmem;
     t->replay[0] = (const void *)k_replay<KMAX, false>;
     t->replay[1] = (const void *)k_replay<KMAX, true>;
     t->replay_per_block = 128;

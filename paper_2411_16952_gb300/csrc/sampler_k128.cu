@@ -694,6 +694,7 @@ void triad_kernels_k128(TriadKernels *t) {
     t->sir[0] = t->sir[1] = nullptr;  // SIR runs use the one-thread form (K <= 64)
     t->refine[0] = (const void *)k_refine_warp<false>;
     t->refine[1] = (const void *)k_refine_warp<true>;
+    t->refine_smem = 0;
     t->replay[0] = (const void *)k_replay_warp<false>;
     t->replay[1] = (const void *)k_replay_warp<true>;
     t->replay_per_block = 32 * kReplayWarps / 32 * kWQ;

@@ -284,7 +284,10 @@ int build_args(tkdv_sampler *h, const unsigned long long *idx0, const unsigned l
     return TKDV_OK;
 }
 
-int refine_grid(tkdv_sampler *h) { return std::max(1, h->num_sms * 4); }
+// CTAs of the FP64 pass.  The one-thread forms' k_refine fills the FP64 pipes
+// with one warp per scheduler, so one CTA of four warps per SM; the warp form's
+// k_refine_warp takes one proposal per warp and four CTAs per SM.
+int refine_grid(tkdv_sampler *h) { return std::max(1, h->num_sms * (h->kt.refine_smem ? 1 : 4)); }
 
 int build_graph(tkdv_sampler *h) {
     if (h->exec) {
@@ -321,6 +324,7 @@ int build_graph(tkdv_sampler *h) {
     rp.func = (void *)h->kt.refine[uni];
     rp.gridDim = dim3(refine_grid(h));
     rp.blockDim = dim3(128);
+    rp.sharedMemBytes = (unsigned)h->kt.refine_smem;
     rp.kernelParams = rargs;
     CK(cudaGraphAddKernelNode(&h->n_refine, h->graph, &h->n_main, 1, &rp));
     CK(cudaGraphInstantiate(&h->exec, h->graph, 0));
@@ -351,6 +355,7 @@ int enqueue(tkdv_sampler *h) {
         rp.func = (void *)h->kt.refine[uni];
         rp.gridDim = dim3(refine_grid(h));
         rp.blockDim = dim3(128);
+        rp.sharedMemBytes = (unsigned)h->kt.refine_smem;
         rp.kernelParams = rargs;
         CK(cudaGraphExecKernelNodeSetParams(h->exec, h->n_refine, &rp));
         CK(cudaGraphLaunch(h->exec, h->stream));
@@ -363,7 +368,7 @@ int enqueue(tkdv_sampler *h) {
     CK(cudaLaunchKernel(main_fn(h, h->launch.variant), dim3(h->launch.ctas), dim3(h->launch.threads), margs,
                         main_dyn_smem(h, h->launch.variant, h->launch.threads), h->stream));
     void *rargs[] = {&h->dev, &h->key0, &h->key1};
-    CK(cudaLaunchKernel(h->kt.refine[uni], dim3(refine_grid(h)), dim3(128), rargs, 0, h->stream));
+    CK(cudaLaunchKernel(h->kt.refine[uni], dim3(refine_grid(h)), dim3(128), rargs, (size_t)h->kt.refine_smem, h->stream));
     return TKDV_OK;
 }
 
@@ -489,6 +494,12 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e != cudaSuccess) {
         h->err = std::string("no CUDA device: ") + cudaGetErrorString(e);
+        return bail(TKDV_ERR_CUDA);
+    }
+    for (int u = 0; u < 2 && h->kt.refine_smem && e == cudaSuccess; ++u)
+        e = cudaFuncSetAttribute(h->kt.refine[u], cudaFuncAttributeMaxDynamicSharedMemorySize, h->kt.refine_smem);
+    if (e != cudaSuccess) {
+        h->err = std::string("FP64 pass shared memory: ") + cudaGetErrorString(e);
         return bail(TKDV_ERR_CUDA);
     }
     // the triad form's accept hand-off may exceed the 48 KB default

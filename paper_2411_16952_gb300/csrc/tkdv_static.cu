@@ -123,6 +123,8 @@ extern "C" int sampler_run_static(int K, const tkdv_point *point, uint64_t idx0,
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e == cudaSuccess && dyn)
         e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess && kt.refine_smem)
+        e = cudaFuncSetAttribute(kt.refine[uni], cudaFuncAttributeMaxDynamicSharedMemorySize, kt.refine_smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, 256, dyn);
     if (e != cudaSuccess) return TKDV_ERR_CUDA;
     const int ctas = std::max(1, nb) * sms;
@@ -164,7 +166,7 @@ extern "C" int sampler_run_static(int K, const tkdv_point *point, uint64_t idx0,
         e = cudaLaunchKernel(fn, dim3(ctas), dim3(256), margs, dyn, st);
         if (e == cudaSuccess) {
             void *rargs[] = {&B, &k0, &k1};
-            e = cudaLaunchKernel(kt.refine[uni], dim3(sms * 4), dim3(128), rargs, 0, st);
+            e = cudaLaunchKernel(kt.refine[uni], dim3(kt.refine_smem ? sms : sms * 4), dim3(128), rargs, (size_t)kt.refine_smem, st);
         }
         if (e != cudaSuccess) return TKDV_ERR_CUDA;
     }
