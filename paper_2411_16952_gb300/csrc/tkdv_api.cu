@@ -94,8 +94,8 @@ int kmax_for(int K) {
     return 0;
 }
 
-// Per-point precompute and the constant table of one point.
-int build_point(tkdv_sampler *h, int p, std::string &msg) {
+// Checks of one point, its alpha* and its proposal variances.
+int check_point(tkdv_sampler *h, int p, std::string &msg) {
     const tkdv_point &q = h->pts[p];
     const int K = h->K;
     if (!(q.E0 > 0) || !std::isfinite(q.E0)) {
@@ -131,25 +131,58 @@ int build_point(tkdv_sampler *h, int p, std::string &msg) {
             return rc;
         }
     }
-    double lm = q.logM;
-    if (!q.override_logM) {
-        int rc = tkdv_log_M(K, q.beta_p, q.E0, q.r, q.proposal == TKDV_PROPOSAL_UNIFORM ? nullptr : s2.data(),
-                            &lm);
-        if (rc != TKDV_OK) {
-            msg = "point " + std::to_string(p) + ": envelope search failed";
-            return rc;
-        }
-    } else if (!std::isfinite(lm)) {
+    if (q.override_logM && !std::isfinite(q.logM)) {
         msg = "point " + std::to_string(p) + ": overridden log M is not finite";
         return TKDV_ERR_INVALID_ARG;
     }
     h->alpha[p] = alpha;
-    h->logM[p] = lm;
     h->sigma2[p] = s2;
+    return TKDV_OK;
+}
 
-    fill_point_const(K, q, s2.data(), lm, false, h->pc_triad[p]);
-    fill_point_const(K, q, s2.data(), lm, true, h->pc_grid[p]);
-    h->pc[p] = h->opt.h3_mode == TKDV_H3_GRID_BF16X3 ? h->pc_grid[p] : h->pc_triad[p];
+// log M of every point that does not bring its own: by the device search
+// (envelope.cu), scratch being a device buffer that holds it, or without a
+// device (scratch null) by tkdv_log_M.
+int find_envelopes(tkdv_sampler *h, void *scratch, std::string &msg) {
+    const int K = h->K;
+    std::vector<int> need;
+    for (int p = 0; p < h->n_points; ++p) {
+        h->logM[p] = h->pts[p].logM;
+        if (!h->pts[p].override_logM) need.push_back(p);
+    }
+    if (need.empty()) return TKDV_OK;
+    const size_t n = need.size();
+    if (scratch) {
+        std::vector<EnvPoint> ep(n);
+        for (size_t i = 0; i < n; ++i) {
+            const tkdv_point &q = h->pts[need[i]];
+            const double K2 = (double)K * K, c = std::sqrt(q.E0 / (2.0 * M_PI));
+            ep[i].cS = -q.beta_p / K2;
+            ep[i].cH = std::fabs(q.beta_p * q.r / (q.E0 * K2) * 2.0 * M_PI * c * c * c);
+            ep[i].cQ = q.proposal == TKDV_PROPOSAL_UNIFORM ? 0.0 : (double)K;
+            for (int k = 0; k < kKMax; ++k) ep[i].w[k] = k < K ? 1.0 / h->sigma2[need[i]][k] : 0.0;
+        }
+        unsigned long long *best = (unsigned long long *)scratch;
+        EnvPoint *d_ep = (EnvPoint *)((char *)scratch + sizeof(unsigned long long) * kMaxPoints);
+        std::vector<unsigned long long> keys(n);
+        CK(cudaMemset(best, 0, sizeof(unsigned long long) * n));
+        CK(cudaMemcpy(d_ep, ep.data(), sizeof(EnvPoint) * n, cudaMemcpyHostToDevice));
+        CK(launch_envelope(d_ep, (int)n, K, best, nullptr));
+        CK(cudaMemcpy(keys.data(), best, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost));
+        for (size_t i = 0; i < n; ++i) h->logM[need[i]] = envelope_value(keys[i]);
+    } else {
+        for (int p : need) {
+            const tkdv_point &q = h->pts[p];
+            if (tkdv_log_M(K, q.beta_p, q.E0, q.r, q.proposal == TKDV_PROPOSAL_UNIFORM ? nullptr : h->sigma2[p].data(),
+                           &h->logM[p]) != TKDV_OK)
+                h->logM[p] = NAN;
+        }
+    }
+    for (int p : need)
+        if (!std::isfinite(h->logM[p])) {
+            msg = "point " + std::to_string(p) + ": envelope search failed";
+            return TKDV_ERR_ENVELOPE;
+        }
     return TKDV_OK;
 }
 
@@ -469,7 +502,7 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
     h->all_uniform = true;
     for (int p = 0; p < n_points; ++p) {
         std::string msg;
-        int rc = build_point(h, p, msg);
+        int rc = check_point(h, p, msg);
         if (rc) {
             delete h;
             return fail(nullptr, rc, msg);
@@ -493,8 +526,10 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
     cudaError_t e = cudaGetDevice(&h->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e != cudaSuccess) {
-        h->err = std::string("no CUDA device: ") + cudaGetErrorString(e);
-        return bail(TKDV_ERR_CUDA);
+        std::string msg;
+        const int rce = find_envelopes(h, nullptr, msg);
+        h->err = rce ? msg : std::string("no CUDA device: ") + cudaGetErrorString(e);
+        return bail(rce ? rce : TKDV_ERR_CUDA);
     }
     for (int u = 0; u < 2 && h->kt.refine_smem && e == cudaSuccess; ++u)
         e = cudaFuncSetAttribute(h->kt.refine[u], cudaFuncAttributeMaxDynamicSharedMemorySize, h->kt.refine_smem);
@@ -546,7 +581,6 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
             grid_kernels_k64(&h->kg);
         h->grid_ok = true;
         h->launch.form = TKDV_H3_GRID_BF16X3;
-        h->pc = h->pc_grid;
         const size_t btile = (size_t)(gridN / 2) * h->kg.ka * 2, atile = (size_t)128 * h->kg.ka * 2;
         // a variant fits if its warpgroups' accumulators (N columns each) fit
         // the 512 TMEM columns of an SM and its tiles the shared memory
@@ -616,6 +650,18 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
         }
         h->own_stream = true;
     }
+    {
+        std::string msg;
+        if ((rc = find_envelopes(h, h->d_refine, msg))) {  // the queue is free before the first run
+            if (!msg.empty()) h->err = msg;
+            return bail(rc);
+        }
+    }
+    for (int p = 0; p < n_points; ++p) {
+        fill_point_const(h->K, h->pts[p], h->sigma2[p].data(), h->logM[p], false, h->pc_triad[p]);
+        fill_point_const(h->K, h->pts[p], h->sigma2[p].data(), h->logM[p], true, h->pc_grid[p]);
+    }
+    h->pc = h->launch.form == TKDV_H3_GRID_BF16X3 ? h->pc_grid : h->pc_triad;
     e = cudaMemcpy(h->d_pts, h->pc.data(), sizeof(PointConst) * n_points, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(h->d_stats, 0, sizeof(StatBlock) * n_points);
     if (e == cudaSuccess) e = cudaMemset(h->d_ring_count, 0, 8);

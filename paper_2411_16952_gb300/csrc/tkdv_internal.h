@@ -188,6 +188,16 @@ inline size_t record_bytes(int K) {
     return (b + 15) & ~(size_t)15;
 }
 
+// One point of the envelope search on the device (envelope.cu): log f/g =
+// cS S + cH T + cQ ln Q over real amplitudes, cH >= 0 (see there).
+struct EnvPoint {
+    double cS, cH, cQ;
+    double w[kKMax];  // 1/sigma_k^2
+};
+// log M of P points of K modes into best (device, zeroed: order-preserving
+// keys, envelope_value gives the number).
+cudaError_t launch_envelope(const EnvPoint *pts, int P, int K, unsigned long long *best, cudaStream_t st);
+double envelope_value(unsigned long long key);
 // Host: proposal variances sigma_k^2 (Eq. 25, learned corrections applied)
 // and alpha*; returns a TKDV_ status.  s2 has K entries.
 int proposal_variances(int K, const tkdv_point &q, double *alpha, double *s2);
