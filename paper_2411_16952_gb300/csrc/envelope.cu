@@ -19,7 +19,7 @@
 // schedulers for eight points at 64 modes), so the search of a handle takes
 // about as long as its slowest start: 0.8 ms for eight points at 64 modes
 // (25 evaluations a start on average), 6 ms for 32 points at 32 modes over two
-// decades of beta', 11 ms for eight at 128 modes, where tkdv_log_M takes 107,
+// decades of beta', 1.9 ms for eight at 128 modes, where tkdv_log_M takes 107,
 // 17 and 830 ms for each point on one host core.  A bisection step of eight
 // 64-mode candidates went from 854 to 8.0 ms, a batch of 32 points at 32 modes
 // from 541 to 14.1 ms, sampling included.
@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(32 * kEnvWarps) k_envelope(const EnvPoint *pts
                 break;
             }
             t *= 0.5;
+            if (t * slope < 1e-16 * scale) break;  // below the noise of F (halving on: 310 evaluations, not 48)
         }
         if (!ok) break;
         double sy = 0.0, ny = 0.0;
