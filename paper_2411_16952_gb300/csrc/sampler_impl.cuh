@@ -70,6 +70,46 @@ struct PhiloxRow {
     __device__ __forceinline__ uint4 block(uint32_t j) const { return philox4x32_10_rk(make_uint4(j, lo, hi, pid), rk); }
 };
 
+// The first three rounds of the blocks (j, lo, hi, pid) of a run share most of
+// their work: with R0..R2 written out, everything that does not depend on lo
+// gives four words per (j, hi, pid, key) (PhiloxHead), and what does not depend
+// on j one product per proposal (PhiloxTail), so a block takes 15 wide products
+// and 17 xors instead of 20 and 20.
+struct PhiloxHead {
+    uint32_t a, b, c, d;
+};
+__device__ __forceinline__ PhiloxHead philox_head(uint32_t j, uint32_t hi, uint32_t pid, const uint32_t *rk) {
+    const unsigned long long p0 = (unsigned long long)j * 0xD2511F53ull, q0 = (unsigned long long)hi * 0xCD9E8D57ull;
+    const uint32_t z1 = (uint32_t)(p0 >> 32) ^ pid ^ rk[1];
+    const unsigned long long q1 = (unsigned long long)z1 * 0xCD9E8D57ull;
+    const uint32_t x2 = (uint32_t)(q1 >> 32) ^ (uint32_t)q0 ^ rk[2];
+    const unsigned long long p2 = (unsigned long long)x2 * 0xD2511F53ull;
+    return {(uint32_t)p0 ^ rk[3], (uint32_t)q1 ^ rk[4], (uint32_t)(p2 >> 32) ^ rk[5], (uint32_t)p2};
+}
+struct PhiloxTail {
+    uint32_t ph, pl;  // M0 x1, x1 the first word after round 0
+    const uint32_t *rk;
+    __device__ __forceinline__ PhiloxTail(uint32_t lo, uint32_t hi, const uint32_t *rk_) : rk(rk_) {
+        const uint32_t x1 = __umulhi(0xCD9E8D57u, hi) ^ lo ^ rk[0];
+        const unsigned long long p = (unsigned long long)x1 * 0xD2511F53ull;
+        ph = (uint32_t)(p >> 32);
+        pl = (uint32_t)p;
+    }
+    // the block of the head's j
+    __device__ __forceinline__ uint4 block(const PhiloxHead &h) const {
+        const unsigned long long q = (unsigned long long)(ph ^ h.a) * 0xCD9E8D57ull;
+        uint4 c = make_uint4((uint32_t)(q >> 32) ^ h.b, (uint32_t)q, pl ^ h.c, h.d);
+#pragma unroll
+        for (int r = 3; r < 10; ++r) {
+            const unsigned long long p0 = (unsigned long long)c.x * 0xD2511F53ull;
+            const unsigned long long p1 = (unsigned long long)c.z * 0xCD9E8D57ull;
+            c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ rk[2 * r], (uint32_t)p1,
+                           (uint32_t)(p0 >> 32) ^ c.w ^ rk[2 * r + 1], (uint32_t)p0);
+        }
+        return c;
+    }
+};
+
 // one_m(w): the float 1 + (w >> 9) 2^-23, i.e. the bits 0x3f800000 | (w >> 9),
 // by one funnel shift of (127 : w) right by 9.
 __device__ __forceinline__ float one_m(uint32_t w) { return __uint_as_float(__funnelshift_r(w, 0x7Fu, 9)); }
@@ -544,6 +584,12 @@ __device__ __forceinline__ void write_record(unsigned char *rec, unsigned long l
     }
 }
 
+// __float2ll_rn, which runs on the FP64 pipe (64 cycles of its scheduler per
+// warp), by the 32-bit conversion where the value fits.
+__device__ __forceinline__ long long fixed_ll(float v) {
+    return fabsf(v) < 2147483520.f ? (long long)__float2int_rn(v) : __float2ll_rn(v);
+}
+
 // Statistics of one accepted draw into the CTA's shared-memory partials.  Out
 // of line: accepted draws are rare, and keeping this code out of the hot loop
 // keeps that loop's instruction-cache footprint small.
@@ -552,10 +598,10 @@ static __device__ __noinline__ void tally_accepted(float u0, float ha, float hb,
     atomicAdd(&s_hist[hist_bin(u0, ha, hb)], 1u);
     atomicAdd(&s_exc[exc_bin(u0, ea)], 1u);
     const float u2 = u0 * u0;
-    atomicAdd(&s_q[0], (unsigned long long)__float2ll_rn(u0 * kQ1));
-    atomicAdd(&s_q[1], (unsigned long long)__float2ll_rn(u2 * kQ2));
-    atomicAdd(&s_q[2], (unsigned long long)__float2ll_rn(u2 * u0 * kQ3));
-    atomicAdd(&s_q[3], (unsigned long long)__float2ll_rn(u2 * u2 * kQ4));
+    atomicAdd(&s_q[0], (unsigned long long)fixed_ll(u0 * kQ1));
+    atomicAdd(&s_q[1], (unsigned long long)fixed_ll(u2 * kQ2));
+    atomicAdd(&s_q[2], (unsigned long long)fixed_ll(u2 * u0 * kQ3));
+    atomicAdd(&s_q[3], (unsigned long long)fixed_ll(u2 * u2 * kQ4));
 }
 
 // Power spectrum of an accepted draw (mean of s_k = xh_k^2 + xh_{K+k}^2 over

@@ -10,186 +10,284 @@
 // pairs (x_m, y_m) to shared memory and keeps its share of |x|^2, S|x|^2,
 // Q|x|^2, u(0) and the smallest radius word, which warp reductions complete.
 //
-// The double sum, for v_k = x_k - i y_k,
-//   T = sum_{k, l >= 1, k + l <= K} Re(v_k v_l conj(v_{k+l})),
-// is cut into 8 x 8 tiles of (k, l) pairs over blocks kb <= lb of eight
-// modes: a tile with kb < lb stands for (k, l) and (l, k) and has weight 2;
-// a diagonal tile holds all ordered pairs of its block and has weight 1.  The
-// 72 tiles with kb + lb <= 15 hold every pair with k + l <= 128; modes above
-// K read as zero, which removes the pairs with k + l > K.  A batch has
-// 4 x 72 = 288 tiles, nine rounds of one tile per lane with every lane on the
-// same instruction stream.  A tile loads its 8 + 8 modes and the 15 sums
-// k + l, sums the products of each anti-diagonal i + j = d in packed FP32
-//   P1 = sum (x_k x_l, y_k y_l),  P2 = sum (y_k x_l, x_k y_l)
-// and weights them by v_{k+l} once per anti-diagonal.  Every term passes
-// through at most 50 roundings (8 in P, 31 in the tile, 3 over rounds, 5 in
-// the warp reduction, 3 in the scaling), within the chain of 64 the decision
-// guard of point_table.cpp allows the warp form, so the guard band and the
+// H3 is the grid cubature of Eq. (2) by a fast transform in FP32, eight lanes
+// per proposal.  With C(xi) = sum x_k cos k xi and S(xi) = sum y_k sin k xi the
+// field at +-xi is proportional to C +- S, and a pair of points contributes
+// 2 C (C^2 + 3 S^2).  2 (C + i S) = sum_k (x_k + y_k) e^{ik xi} + (x_k - y_k)
+// e^{-ik xi} has real coefficients c_k, k = 1..128 and -1..-128, so on the
+// N = 384 points xi_j = 2 pi (j + 1/2)/N the points j and N - 1 - j are
+// conjugate and N/2 = 192 values suffice.  With k = k1 + 24 k2 and j = j2 + 16
+// j1 (j2 even: one of each conjugate pair)
+//   value_j = sum_{k1} e^{2 pi i k1 j1/24} [e^{i pi k1 (2 j2 + 1)/384}
+//             sum_{k2} c_{k1 + 24 k2} e^{2 pi i k2 (j2 + 1/2)/16}];
+// the inner sum over 16 real c, X_n and X_{n+8} joined to X_n + i X_{n+8}, is
+// an 8-point transform of (X_n + i X_{n+8}) e^{2 pi i n/32}, whose results are
+// j2 = 0, 2, .., 14.  A lane makes three of the 24 columns k1, twists and
+// stores them, and takes one j2: 24 = 3 x 8 points without further twists
+// (3 and 8 have no common factor), cubed and summed as they come.  N = 384 =
+// 3 x 128 points do not integrate e^{+-i 384 xi}: the cube of mode 128 alone
+// aliases, and its term (N/4) Re v_128^3, with the sign of the half-step
+// offset, is added back.
+//
+// What bounds it: issue of the FP32 and integer pipes.  The transform is about
+// 6,400 thread instructions per proposal; 8 x 8 tiles of the double sum of
+// Eq. (42), the form before, took 26,000 (4608 packed products of 2 cycles
+// each, their loads and the tiles' ends), of 33,300 in all; now 20,100 in all,
+// issue 75 % busy (60 % before).  2 x 2^21 proposals at acceptance 0.28: 6.58 ms
+// with the tiles, 3.90 ms with the transform, 3.43 ms with the draw loop rolled
+// up, the shared Philox rounds, and the spectrum of accepted draws in
+// registers (64-bit float conversions run on the FP64 pipe, 12 % busy with
+// them).  The transform's error in H3 against FP64, with that of the draw, is
+// 4.8e-7 of the root mean square (3.8e-7 with the tiles; nearly all of the
+// difference to log f/(Mg), 1.2e-5, is the draw's and unchanged).
+//
+// Rounding: the 2-norm of the 192 values is off by at most 25 roundings
+// (coefficients 1, three-level 8-point transforms 5 each, twists 3 each, the
+// 3-point one 3), which moves T by 2 sqrt(K) of it, and the sum of the cubes
+// adds chains of at most 13 terms: 75 2^-24 sqrt(K), against the 512 2^-24
+// sqrt(K) of the decision guard of point_table.cpp, so the guard band and the
 // FP64 pass (k_refine_warp) keep every accept decision exact.  The radius is
 // rho_log, the full-precision logarithm, whose error is purely relative: the
 // guard needs no per-draw radius terms and is about ten times narrower than
 // it would be with the fast radius, so that about 0.15 % of the draws at
 // K = 128 reach the FP64 pass.
 //
-// Shared-memory layout: proposal q of a warp at word q * kWS, mode m at word
-// m + m/8 (one pad word per block of eight), so that lanes reading the same
-// mode of consecutive blocks hit distinct banks.  Modes K..135 stay zero.
+// Shared memory of a warp: proposal q's state at float2 word q * kWS, mode m
+// (from 0) at word m, modes K..127 zero; then its transform at q * kWB, value
+// (l, k1) at word kWR l + k1.  The strides put the eight lanes of the two
+// proposals of a half-warp on distinct banks in every access.
 #include "sampler_impl.cuh"
 
 namespace tkdv {
 namespace {
 
-constexpr int kWK = 128;                      // modes of the layout
-constexpr int kWQ = 4;                        // proposals per warp batch
-constexpr int kWS = 153;                      // float2 words per proposal (mode 135 at word 151)
-constexpr int kWTiles = 72;                   // tiles per proposal
-constexpr int kWRounds = kWQ * kWTiles / 32;  // tile rounds per batch (9)
-static_assert(kWQ * kWTiles == 32 * kWRounds, "tiles must fill whole rounds");
+constexpr int kWK = 128;  // modes of the layout
+constexpr int kWQ = 4;    // proposals per warp batch, eight lanes each
+constexpr int kWN = 384;  // grid points
+constexpr int kWS = 136;  // float2 words of one proposal's state
+constexpr int kWR = 25;   // float2 words of one row (24 columns) of the transform
+constexpr int kWB = 8 * kWR;  // float2 words of one proposal's transform
+constexpr int kWarpWords = kWQ * (kWS + kWB);  // float2 words of a warp's slab
 
-__device__ __forceinline__ int wpos(int m) { return m + (m >> 3); }
+struct cf {
+    float x, y;
+};
+__device__ __forceinline__ cf operator+(cf a, cf b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ cf operator-(cf a, cf b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ cf cmul(cf a, float c, float s) {
+    return {fmaf(a.x, c, -(a.y * s)), fmaf(a.x, s, a.y * c)};
+}
+__device__ __forceinline__ cf muli(cf a) { return {-a.y, a.x}; }
 
-// Tile t of a batch: proposal q = t / 72 and the (kb, lb) pair number t % 72
-// in the order kb = 0..7, lb = kb..15-kb.  x: word offsets of the k and l
-// blocks; y: word offset of block kb + lb, q << 16, weight << 24.
-__device__ uint2 tile_entry(int t) {
-    const int q = t / kWTiles;
-    int f = t % kWTiles, kb = 0;
-    while (f >= 16 - 2 * kb) {
-        f -= 16 - 2 * kb;
-        ++kb;
-    }
-    const int lb = kb + f;
-    const uint32_t base = (uint32_t)(q * kWS);
-    uint2 e;
-    e.x = (base + 9u * kb) | ((base + 9u * lb) << 16);
-    e.y = (base + 9u * (kb + lb)) | ((uint32_t)q << 16) | ((kb < lb ? 2u : 1u) << 24);
-    return e;
+// z_k = sum_n z_n e^{2 pi i n k/8}, in place.
+__device__ __forceinline__ void dft8(cf *z) {
+    constexpr float r = 0.70710678118654752440f;
+    const cf a0 = z[0] + z[4], a1 = z[0] - z[4], a2 = z[2] + z[6], a3 = muli(z[2] - z[6]);
+    const cf b0 = z[1] + z[5], b1 = z[1] - z[5], b2 = z[3] + z[7], b3 = muli(z[3] - z[7]);
+    const cf e0 = a0 + a2, e2 = a0 - a2, e1 = a1 + a3, e3 = a1 - a3;
+    const cf o0 = b0 + b2, o2 = muli(b0 - b2), o1 = b1 + b3, o3 = b1 - b3;
+    z[0] = e0 + o0;
+    z[4] = e0 - o0;
+    z[2] = e2 + o2;
+    z[6] = e2 - o2;
+    // e^{i pi/4} o1 = r (o1.x - o1.y, o1.x + o1.y);  e^{3 i pi/4} o3 = r (-o3.x - o3.y, o3.x - o3.y)
+    const float u = o1.x - o1.y, v = o1.x + o1.y, p = o3.x + o3.y, q = o3.x - o3.y;
+    z[1] = {fmaf(r, u, e1.x), fmaf(r, v, e1.y)};
+    z[5] = {fmaf(-r, u, e1.x), fmaf(-r, v, e1.y)};
+    z[3] = {fmaf(-r, p, e3.x), fmaf(r, q, e3.y)};
+    z[7] = {fmaf(r, p, e3.x), fmaf(-r, q, e3.y)};
 }
 
-// sum over the tile's pairs of Re(v_k v_l conj(v_{k+l})), unweighted.
-__device__ __forceinline__ float tile_sum(const float2 *sv, uint32_t ko, uint32_t lo, uint32_t no) {
-    f32x2_t A[8], As[8], Bv[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float2 a = sv[ko + i];
-        A[i] = pk2(a.x, a.y);
-        As[i] = pk2(a.y, a.x);
+// Twist of value (l, k1): e^{2 pi i k1 (4 l + 1)/768}, at word 24 l + k1.
+__device__ __forceinline__ float2 twist_entry(int t) {
+    const int l = t / 24, k1 = t % 24;
+    float sn, cs;
+    sincospif((float)(k1 * (4 * l + 1)) / 384.f, &sn, &cs);
+    return make_float2(cs, sn);
+}
+
+// Column k1 = 8 C + s of a proposal: its 16 coefficients c_{k1 + 24 k2} (k <=
+// 128 positive, k >= 256 standing for k - 384 with the sign of the half step), the 8-point transform, the
+// twists, and the results to the rows l = 0..7 of wt.
+template <int C>
+__device__ __forceinline__ void column(const float2 *sv, float2 *wt, const float2 *tw, int s) {
+    const int k1 = 8 * C + s;
+    auto pos = [&](int k2) {  // x + y of mode k1 + 24 k2
+        const float2 v = sv[k1 + 24 * k2 - 1];
+        return v.x + v.y;
+    };
+    auto neg = [&](int k2) {  // -(x - y) of mode 384 - k1 - 24 k2: e^{-384 i xi_j} = -1
+        const float2 v = sv[kWN - k1 - 24 * k2 - 1];
+        return v.y - v.x;
+    };
+    // e^{2 pi i n/32}, n = 1..7
+    constexpr float c1 = 0.98078528040323044913f, s1 = 0.19509032201612826785f, c2 = 0.92387953251128675613f,
+                    s2 = 0.38268343236508977173f, c3 = 0.83146961230254523708f, s3 = 0.55557023301960222474f,
+                    c4 = 0.70710678118654752440f;
+    cf z[8];
+    z[0] = {C > 0 || s > 0 ? pos(0) : 0.f, 0.f};  // (k = 0 has no mode)
+    const float x1 = pos(1);
+    z[1] = {x1 * c1, x1 * s1};
+    const float x2 = pos(2);
+    if (C == 2) {
+        z[2] = cmul({x2, neg(10)}, c2, s2);  // k = 240 + k1 >= 256
+    } else {
+        z[2] = {x2 * c2, x2 * s2};
     }
+    z[3] = cmul({pos(3), neg(11)}, c3, s3);
+    z[4] = cmul({pos(4), neg(12)}, c4, c4);
+    // k = 120 + k1 <= 128: all of column block 0, the first of block 1
+    const float x5 = C == 0 ? pos(5) : C == 1 && s == 0 ? pos(5) : 0.f;
+    z[5] = cmul({x5, neg(13)}, s3, c3);
+    const float x6 = neg(14), x7 = neg(15);
+    z[6] = {-x6 * c2, x6 * s2};  // i x6 e^{2 pi i 6/32}
+    z[7] = {-x7 * c1, x7 * s1};  // i x7 e^{2 pi i 7/32}
+    dft8(z);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const float2 b = sv[lo + j];
-        Bv[j] = pk2(b.x, b.y);
+    for (int l = 0; l < 8; ++l) {
+        const float2 t = tw[24 * l + k1];
+        const cf v = cmul(z[l], t.x, t.y);
+        wt[kWR * l + k1] = make_float2(v.x, v.y);
     }
-    f32x2_t P1[15], P2[15];
+}
+
+// sum of C (C^2 + 3 S^2) over the 24 points of row l = s.
+__device__ __forceinline__ float row_cubes(const float2 *wr) {
+    constexpr float h = 0.86602540378443864676f;
+    cf z[3][8];
 #pragma unroll
-    for (int d = 0; d < 15; ++d) P1[d] = P2[d] = 0ull;
+    for (int a = 0; a < 8; ++a) {
+        const float2 v0 = wr[(3 * a) % 24], v1 = wr[(3 * a + 8) % 24], v2 = wr[(3 * a + 16) % 24];
+        const cf sm = {v1.x + v2.x, v1.y + v2.y}, d = {v1.x - v2.x, v1.y - v2.y};
+        z[0][a] = {v0.x + sm.x, v0.y + sm.y};
+        const cf t = {fmaf(-0.5f, sm.x, v0.x), fmaf(-0.5f, sm.y, v0.y)};
+        z[1][a] = {fmaf(-h, d.y, t.x), fmaf(h, d.x, t.y)};
+        z[2][a] = {fmaf(h, d.y, t.x), fmaf(-h, d.x, t.y)};
+    }
+    float acc[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int b = 0; b < 3; ++b) {
+        dft8(z[b]);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            P1[i + j] = fma2(A[i], Bv[j], P1[i + j]);
-            P2[i + j] = fma2(As[i], Bv[j], P2[i + j]);
+            const float c2 = z[b][j].x * z[b][j].x, s2 = z[b][j].y * z[b][j].y;
+            acc[b] = fmaf(z[b][j].x, fmaf(3.f, s2, c2), acc[b]);
         }
     }
-    float t = 0.f;
-#pragma unroll
-    for (int d = 0; d < 15; ++d) {
-        // k + l = 8 (kb + lb) + d + 2, i.e. mode 8 (kb + lb) + d + 1
-        const float2 vn = sv[no + (d + 1) + ((d + 1) >> 3)];
-        float a0, a1, b0, b1;
-        upk2(P1[d], a0, a1);
-        upk2(P2[d], b0, b1);
-        t = fmaf(vn.x, a0 - a1, t);
-        t = fmaf(vn.y, b0 + b1, t);
-    }
-    return t;
-}
-
-__device__ __forceinline__ float wsum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;  // the same value in every lane (each level adds a commuting pair)
-}
-
-__device__ __forceinline__ float sel4(const float *a, int q) {
-    return q == 0 ? a[0] : q == 1 ? a[1] : q == 2 ? a[2] : a[3];
+    return (acc[0] + acc[1]) + acc[2];
 }
 
 // One batch of the fast path: the four proposals' draws, reductions and T.
 // On return every lane holds the values of proposal ql = lane & 3.
 struct WEval {
     float nrm2, Sraw, zz, u0raw, T;
-    uint32_t wmin;
+    bool tail;  // a radius word in the lowest bucket of the uniform map
 };
 
-template <bool UNIF>
-__device__ __forceinline__ WEval warp_batch(float2 *sv, const uint2 *s_tab, const float *sig, const float *act,
-                                            int K, const uint32_t *lo, const uint32_t *hi, uint32_t vmask,
-                                            uint32_t pid, uint32_t k0, uint32_t k1, int lane) {
-    float nrm2[kWQ], Sraw[kWQ], zz[kWQ], u0raw[kWQ];
-    uint32_t wmin[kWQ];
-#pragma unroll
-    for (int q = 0; q < kWQ; ++q) {
-        nrm2[q] = Sraw[q] = zz[q] = u0raw[q] = 0.f;
-        wmin[q] = 0xFFFFFFFFu;
+// The lane's two Philox blocks (lane and lane + 32): their heads for the index
+// half `hi` they were made for.
+struct WHeads {
+    PhiloxHead h[2];
+    uint32_t hi;
+    __device__ __forceinline__ void make(uint32_t hi_, uint32_t pid, const uint32_t *rk, int lane) {
+        hi = hi_;
+        h[0] = philox_head((uint32_t)lane, hi, pid, rk);
+        h[1] = philox_head((uint32_t)lane + 32u, hi, pid, rk);
     }
+};
+
+// idx(q): the index of the batch's proposal q, q in vmask.
+template <bool UNIF, typename Idx>
+__device__ __forceinline__ WEval warp_batch(float2 *sv, const float2 *s_tw, const float *sig, const float *act, int K,
+                                            const Idx &idx, uint32_t vmask, WHeads &heads, uint32_t pid,
+                                            const uint32_t *rk, int lane) {
+    uint32_t tails = 0;
     // Steps 1-3: lane L makes the Philox blocks L and L + 32 of every proposal.
     // The radius is rho_log (purely relative error), so the outputs of
-    // accepted draws need no second pass and the guard no per-draw terms.
+    // accepted draws need no second pass and the guard no per-draw terms.  The
+    // loop stays rolled: with the four proposals written out the loop body
+    // (about 3,000 instructions) missed the instruction cache 1.2 times an
+    // issue.  Partial sums |x|^2, S|x|^2, Q|x|^2 and u(0)|x|/u0s go to the
+    // words of the transform, [q][lane] in steps of 4, 136 apart.
+    float *part = reinterpret_cast<float *>(sv + kWQ * kWS);
+#pragma unroll 1
+    for (int q = 0; q < kWQ; ++q) {
+        float nrm2 = 0.f, Sraw = 0.f, zz = 0.f, u0raw = 0.f;
+        if ((vmask >> q) & 1u) {
+            const unsigned long long id = idx(q);
+            if ((uint32_t)(id >> 32) != heads.hi) heads.make((uint32_t)(id >> 32), pid, rk, lane);
+            const PhiloxTail tail((uint32_t)id, heads.hi, rk);
 #pragma unroll
-    for (int i = 0; i < 2 * kWQ; ++i) {
-        const int q = i >> 1;
-        const int j = lane + 32 * (i & 1);
-        if (((vmask >> q) & 1u) && 2 * j < K) {
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)j, lo[q], hi[q], pid), k0, k1);
+            for (int i = 0; i < 2; ++i) {
+                const int j = lane + 32 * i;
+                if (2 * j < K) {
+                    const uint4 w = tail.block(heads.h[i]);
+                    float xy[4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int m = 2 * j + h;
-                const float s = UNIF ? act[m] : sig[m];
-                const float rho = rho_log(h ? w.z : w.x);
-                const float a = (-s * rho) * rsqrt_approx(rho);
-                float sn, cs;
-                sincos_approx(angle_f(h ? w.w : w.y), sn, cs);
-                const float xm = a * cs, ym = a * sn;
-                if (m < K) wmin[q] = min(wmin[q], h ? w.z : w.x);
-                sv[q * kWS + wpos(m)] = make_float2(xm, ym);
-                const float sk = (s * s) * rho;
-                nrm2[q] += sk;
-                Sraw[q] = fmaf((float)((m + 1) * (m + 1)), sk, Sraw[q]);
-                zz[q] += s > 0.f ? rho : 0.f;
-                u0raw[q] += xm;
+                    for (int h = 0; h < 2; ++h) {
+                        const int m = 2 * j + h;
+                        const float s = UNIF ? act[m] : sig[m];
+                        const float rho = rho_log(h ? w.z : w.x);
+                        const float a = (-s * rho) * rsqrt_approx(rho);
+                        float sn, cs;
+                        sincos_approx(angle_f(h ? w.w : w.y), sn, cs);
+                        const float xm = a * cs, ym = a * sn;
+                        if (m < K && (h ? w.z : w.x) < kTailBucket) tails |= 1u << q;
+                        xy[2 * h] = xm;
+                        xy[2 * h + 1] = ym;
+                        const float sk = (s * s) * rho;
+                        nrm2 += sk;
+                        Sraw = fmaf((float)((m + 1) * (m + 1)), sk, Sraw);
+                        zz += s > 0.f ? rho : 0.f;
+                        u0raw += xm;
+                    }
+                    *reinterpret_cast<float4 *>(sv + q * kWS + 2 * j) = make_float4(xy[0], xy[1], xy[2], xy[3]);
+                }
             }
         }
+        *reinterpret_cast<float4 *>(part + q * 136 + 4 * lane) = make_float4(nrm2, Sraw, zz, u0raw);
     }
+    tails = __reduce_or_sync(0xffffffffu, tails);
+    __syncwarp();
+    // The 16 sums over the warp: lanes 2 e and 2 e + 1 take sum e = 4 stat + q,
+    // the partial sums of the even and of the odd lanes, in the order of a
+    // butterfly (lanes 16, 8, 4 and 2 apart, then the two halves).
+    float tot;
+    {
+        const float *src = part + ((lane >> 1) & 3) * 136 + 4 * (lane & 1) + (lane >> 3);
+        float t[8];
 #pragma unroll
-    for (int q = 0; q < kWQ; ++q) {
-        nrm2[q] = wsum(nrm2[q]);
-        Sraw[q] = wsum(Sraw[q]);
-        zz[q] = wsum(zz[q]);
-        u0raw[q] = wsum(u0raw[q]);
-        wmin[q] = __reduce_min_sync(0xffffffffu, wmin[q]);
+        for (int e = 0; e < 8; ++e) t[e] = src[8 * e] + src[8 * (e + 8)];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+            for (int e = 0; e < o; ++e) t[e] += t[e + o];
+        tot = t[0] + __shfl_xor_sync(0xffffffffu, t[0], 1);
     }
     __syncwarp();
-    // Step 4: nine rounds of one tile per lane.
-    float Tq[kWQ] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-    for (int r = 0; r < kWRounds; ++r) {
-        const uint2 e = s_tab[r * 32 + lane];
-        const float t = tile_sum(sv, e.x & 0xFFFFu, e.x >> 16, e.y & 0xFFFFu) * (float)(e.y >> 24);
-        const int q = (int)((e.y >> 16) & 0xFFu);
+    // Step 4: the transform, eight lanes per proposal.
+    const int q = lane >> 3, s = lane & 7;
+    const float2 *xq = sv + q * kWS;
+    float2 *wt = sv + kWQ * kWS + q * kWB;
+    column<0>(xq, wt, s_tw, s);
+    column<1>(xq, wt, s_tw, s);
+    column<2>(xq, wt, s_tw, s);
+    __syncwarp();
+    float cub = row_cubes(wt + kWR * s);
 #pragma unroll
-        for (int qq = 0; qq < kWQ; ++qq) Tq[qq] += q == qq ? t : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < kWQ; ++q) Tq[q] = wsum(Tq[q]);
+    for (int o = 4; o > 0; o >>= 1) cub += __shfl_xor_sync(0xffffffffu, cub, o);
     const int ql = lane & 3;
     WEval ev;
-    ev.nrm2 = sel4(nrm2, ql);
-    ev.Sraw = sel4(Sraw, ql);
-    ev.zz = sel4(zz, ql);
-    ev.u0raw = sel4(u0raw, ql);
-    ev.T = sel4(Tq, ql);
-    ev.wmin = ql == 0 ? wmin[0] : ql == 1 ? wmin[1] : ql == 2 ? wmin[2] : wmin[3];
+    ev.nrm2 = __shfl_sync(0xffffffffu, tot, 2 * ql);
+    ev.Sraw = __shfl_sync(0xffffffffu, tot, 8 + 2 * ql);
+    ev.zz = __shfl_sync(0xffffffffu, tot, 16 + 2 * ql);
+    ev.u0raw = __shfl_sync(0xffffffffu, tot, 24 + 2 * ql);
+    // values and coefficients are 2 (C + i S): sum U^3 = 2 cub/8, less the
+    // alias -(N/4) Re v_128^3, and T |x|^3 = (4/(3N)) sum U^3
+    const float2 e = sv[ql * kWS + kWK - 1];
+    const float alias = e.x * fmaf(e.x, e.x, -3.f * (e.y * e.y));
+    ev.T = fmaf(__shfl_sync(0xffffffffu, cub, 8 * ql), 1.f / (3.f * kWN), alias * (1.f / 3.f));
+    ev.tail = (tails >> ql) & 1u;
     return ev;
 }
 
@@ -212,20 +310,16 @@ __device__ __forceinline__ Fast warp_eval(const WEval &ev, const Scal &c, uint32
     return f;
 }
 
-// Shared state common to the sampler and the replay kernel: tile table,
-// proposal variances and the warps' state slabs (zeroed: modes above K).
-template <int NW>
+// Shared state common to the sampler and the replay kernel: the twists and the
+// proposal variances; the warps' slabs are zeroed (modes above K stay zero).
 struct WShared {
-    uint2 tab[32 * kWRounds];
+    float2 tw[kWB];
     float sig[kWK], act[kWK];
-    float2 v[NW][kWQ * kWS];
 };
 
-template <int NW>
-__device__ void wshared_init(WShared<NW> &sh, int tid, int nt) {
-    for (int t = tid; t < 32 * kWRounds; t += nt) sh.tab[t] = tile_entry(t);
-    float2 *v = &sh.v[0][0];
-    for (int e = tid; e < NW * kWQ * kWS; e += nt) v[e] = make_float2(0.f, 0.f);
+__device__ void wshared_init(WShared &sh, float2 *slabs, int nw, int tid, int nt) {
+    for (int t = tid; t < 8 * 24; t += nt) sh.tw[t] = twist_entry(t);
+    for (int e = tid; e < nw * kWarpWords; e += nt) slabs[e] = make_float2(0.f, 0.f);
 }
 
 // ---- FP64 pass of the warp form -------------------------------------------
@@ -409,7 +503,8 @@ template <bool UNIF, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_sample_warp(const __grid_constant__ DevBufs B, const __grid_constant__ RunArgs A, uint32_t k0, uint32_t k1) {
     constexpr int NW = NT / 32;
-    __shared__ WShared<NW> sh;
+    extern __shared__ __align__(16) float2 s_slabs[];
+    __shared__ WShared sh;
     __shared__ uint32_t s_hist[kHistBins];
     __shared__ uint32_t s_exc[kExcBins];
     __shared__ unsigned long long s_q[4];
@@ -419,7 +514,7 @@ __global__ void __launch_bounds__(NT, MINB)
     __shared__ uint32_t s_chunk;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ql = lane & 3;
-    wshared_init<NW>(sh, tid, NT);
+    wshared_init(sh, s_slabs, NW, tid, NT);
     for (int e = tid; e < kHistBins; e += NT) s_hist[e] = 0;
     for (int e = tid; e < kWK; e += NT) s_spec[e] = 0ull;
     if (tid < kExcBins) s_exc[tid] = 0;
@@ -428,7 +523,7 @@ __global__ void __launch_bounds__(NT, MINB)
         s_cnt[tid] = 0;
     }
     if (tid == 0) s_maxd = 0;
-    float2 *sv = sh.v[warp];
+    float2 *sv = s_slabs + warp * kWarpWords;
     const uint32_t total = A.chunk_prefix[A.n_points];
     const unsigned long long t0 = A.deadline_ns ? globaltimer_ns() : 0ull;
 
@@ -459,22 +554,20 @@ __global__ void __launch_bounds__(NT, MINB)
         __syncthreads();
 
         float maxd = -INFINITY;
+        WHeads heads;
+        heads.make((uint32_t)(base >> 32), sc.pid, A.rk.k, lane);
+        unsigned long long spec[kWK / 32] = {0ull, 0ull, 0ull, 0ull}, qsum[4] = {0ull, 0ull, 0ull, 0ull};
         for (uint32_t i0 = (uint32_t)warp * kWQ; i0 < n_here; i0 += (uint32_t)NW * kWQ) {
-            uint32_t lo[kWQ], hi[kWQ], vmask = 0;
-#pragma unroll
-            for (int q = 0; q < kWQ; ++q) {
-                const unsigned long long idx = base + i0 + q;
-                lo[q] = (uint32_t)idx;
-                hi[q] = (uint32_t)(idx >> 32);
-                if (i0 + q < n_here) vmask |= 1u << q;
-            }
-            const WEval ev = warp_batch<UNIF>(sv, sh.tab, sh.sig, sh.act, sc.K, lo, hi, vmask, sc.pid, k0, k1, lane);
-            const uint32_t lq = ql == 0 ? lo[0] : ql == 1 ? lo[1] : ql == 2 ? lo[2] : lo[3];
-            const uint32_t hq = ql == 0 ? hi[0] : ql == 1 ? hi[1] : ql == 2 ? hi[2] : hi[3];
-            const uint32_t wa = accept_word(lq, hq, sc.pid, sc.K, k0, k1);
+            const uint32_t left_here = n_here - i0, vmask = left_here < kWQ ? (1u << left_here) - 1u : (1u << kWQ) - 1u;
+            const WEval ev = warp_batch<UNIF>(
+                sv, sh.tw, sh.sig, sh.act, sc.K, [&](int q) { return base + i0 + (unsigned)q; }, vmask, heads, sc.pid,
+                A.rk.k, lane);
+            const unsigned long long idx = base + i0 + (unsigned)ql;
+            const uint32_t lq = (uint32_t)idx, hq = (uint32_t)(idx >> 32);
+            const uint32_t wa = PhiloxRow(lq, hq, sc.pid, A.rk.k).block((uint32_t)((sc.K + 1) / 2)).x;
             const Fast f = warp_eval<UNIF>(ev, sc, wa);
             const bool valid = lane < kWQ && ((vmask >> lane) & 1u);
-            const bool tail = min(ev.wmin, wa) < kTailBucket;
+            const bool tail = ev.tail || wa < kTailBucket;
             bool defer = valid && (fabsf(f.d) < f.guard || tail);
             if (valid && !tail) maxd = fmaxf(maxd, f.delta);
 
@@ -503,52 +596,66 @@ __global__ void __launch_bounds__(NT, MINB)
             if (valid && !defer && f.delta > 0.f) atomicAdd(&s_cnt[1], 1u);
 
             unsigned ma = __ballot_sync(0xffffffffu, acc);
-            while (ma) {  // rare: the whole warp writes each accepted record
-                const int q = __ffs(ma) - 1;
-                ma &= ma - 1;
-                const float inv = __shfl_sync(0xffffffffu, f.inv, q);
-                const float u0 = __shfl_sync(0xffffffffu, sc.u0s * ev.u0raw * f.inv, q);
-                unsigned long long slot = 0;
+            if (ma) {
+                // one slot range for the batch; the lane of an accepted draw
+                // tallies u(0) and writes the header, then the warp takes the
+                // draws in turn, four modes per lane, the spectrum summed in
+                // registers until the end of the chunk
+                unsigned long long slot0 = 0;
                 if (lane == 0) {
-                    slot = atomicAdd(B.ring_count, 1ull);
-                    atomicAdd(&s_cnt[0], 1u);
+                    slot0 = atomicAdd(B.ring_count, (unsigned long long)__popc(ma));
+                    atomicAdd(&s_cnt[0], (uint32_t)__popc(ma));
                 }
-                slot = __shfl_sync(0xffffffffu, slot, 0);
-                unsigned char *rec = slot < B.ring_cap ? B.ring + slot * B.rec_bytes : nullptr;
-                const float sc2 = (inv * inv) * kSpecScale;
-                float *xh = rec ? reinterpret_cast<float *>(rec + 32) : nullptr;
-#pragma unroll
-                for (int cc = 0; cc < kWK / 32; ++cc) {
-                    const int m = lane + 32 * cc;
-                    if (m < sc.K) {
-                        const float2 v = sv[q * kWS + wpos(m)];
-                        atomicAdd(&s_spec[m], (unsigned long long)__float2ull_rn(fmaf(v.x, v.x, v.y * v.y) * sc2));
-                        if (xh) {
-                            xh[m] = v.x * inv;
-                            xh[sc.K + m] = v.y * inv;
-                        }
-                    }
-                }
-                if (lane == q) {
-                    tally_accepted(u0, sc.ha, sc.hb, sc.ea, s_hist, s_exc, s_q);
-                    if (rec) {
-                        *reinterpret_cast<unsigned long long *>(rec) = ((unsigned long long)hq << 32) | lq;
-                        uint32_t *h = reinterpret_cast<uint32_t *>(rec + 8);
-                        h[0] = (uint32_t)p;
-                        h[1] = 0u;
-                        float *fr = reinterpret_cast<float *>(rec + 16);
-                        fr[0] = sc.E0 * f.S;
-                        fr[1] = sc.h3s * f.T;
-                        fr[2] = u0;
-                        fr[3] = f.delta;
+                slot0 = __shfl_sync(0xffffffffu, slot0, 0);
+                unsigned char *rec = nullptr;
+                if (acc) {
+                    const float u0 = sc.u0s * ev.u0raw * f.inv, u2 = u0 * u0;
+                    atomicAdd(&s_hist[hist_bin(u0, sc.ha, sc.hb)], 1u);
+                    atomicAdd(&s_exc[exc_bin(u0, sc.ea)], 1u);
+                    qsum[0] += (unsigned long long)fixed_ll(u0 * kQ1);
+                    qsum[1] += (unsigned long long)fixed_ll(u2 * kQ2);
+                    qsum[2] += (unsigned long long)fixed_ll(u2 * u0 * kQ3);
+                    qsum[3] += (unsigned long long)fixed_ll(u2 * u2 * kQ4);
+                    const unsigned long long slot = slot0 + __popc(ma & ((1u << lane) - 1u));
+                    if (slot < B.ring_cap) {
+                        rec = B.ring + slot * B.rec_bytes;
+                        write_header(rec, ((unsigned long long)hq << 32) | lq, (uint32_t)p, 0u, sc.E0 * f.S,
+                                     sc.h3s * f.T, u0, f.delta);
                     } else {
                         atomicAdd(&s_cnt[2], 1u);
                     }
                 }
+                do {
+                    const int q = __ffs(ma) - 1;
+                    ma &= ma - 1;
+                    const float inv = __shfl_sync(0xffffffffu, f.inv, q);
+                    float *xh = reinterpret_cast<float *>(
+                        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(rec), q));
+                    const float sc2 = (inv * inv) * kSpecScale;
+#pragma unroll
+                    for (int cc = 0; cc < kWK / 32; ++cc) {
+                        const int m = lane + 32 * cc;
+                        if (m < sc.K) {
+                            const float2 v = sv[q * kWS + m];
+                            // (below 2^28: the 32-bit conversion; the 64-bit one runs on the FP64 pipe)
+                            spec[cc] += __float2uint_rn(fmaf(v.x, v.x, v.y * v.y) * sc2);
+                            if (xh) {
+                                xh[8 + m] = v.x * inv;
+                                xh[8 + sc.K + m] = v.y * inv;
+                            }
+                        }
+                    }
+                } while (ma);
             }
             __syncwarp();  // the next batch overwrites the slab
         }
         // chunk done: flush this CTA's partials into the point's StatBlock
+#pragma unroll
+        for (int cc = 0; cc < kWK / 32; ++cc)
+            if (spec[cc]) atomicAdd(&s_spec[lane + 32 * cc], spec[cc]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (qsum[e]) atomicAdd(&s_q[e], qsum[e]);
         uint32_t key = fkey(maxd);
         key = __reduce_max_sync(0xffffffffu, key);
         if (lane == 0 && maxd > -INFINITY) atomicMax(&s_maxd, key);
@@ -597,10 +704,10 @@ template <bool UNIF>
 __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointConst *P, const unsigned long long *idx,
                                                                    unsigned long long n, uint32_t k0, uint32_t k1,
                                                                    double *out) {
-    __shared__ WShared<kReplayWarps> sh;
-    __shared__ double2 s_x[kReplayWarps][kWK];
+    __shared__ WShared sh;
+    __shared__ __align__(16) float2 s_slabs[kReplayWarps * kWarpWords];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ql = lane & 3;
-    wshared_init<kReplayWarps>(sh, tid, 32 * kReplayWarps);
+    wshared_init(sh, s_slabs, kReplayWarps, tid, 32 * kReplayWarps);
     for (int e = tid; e < kWK; e += 32 * kReplayWarps) {
         sh.sig[e] = P->sigma[e];
         sh.act[e] = P->act[e];
@@ -610,23 +717,27 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
     const int K = sc.K;
     const unsigned long long b0 = ((unsigned long long)blockIdx.x * kReplayWarps + warp) * kWQ;
     if (b0 >= n) return;  // whole warps leave together
-    float2 *sv = sh.v[warp];
-    uint32_t lo[kWQ], hi[kWQ], vmask = 0;
+    float2 *sv = s_slabs + warp * kWarpWords;
+    // the FP64 state of a proposal takes the place of the transform
+    double2 *sx = reinterpret_cast<double2 *>(sv + kWQ * kWS);
+    static_assert(sizeof(double2) * kWK <= sizeof(float2) * kWQ * kWB, "the FP64 state fits the transform's words");
+    const uint32_t vmask = n - b0 < kWQ ? (1u << (n - b0)) - 1u : (1u << kWQ) - 1u;
+    uint32_t rk[20];
 #pragma unroll
-    for (int q = 0; q < kWQ; ++q) {
-        const unsigned long long i = b0 + q < n ? b0 + q : n - 1;
-        const unsigned long long id = idx[i];
-        lo[q] = (uint32_t)id;
-        hi[q] = (uint32_t)(id >> 32);
-        if (b0 + q < n) vmask |= 1u << q;
+    for (int r = 0; r < 10; ++r) {
+        rk[2 * r] = k0 + (uint32_t)r * 0x9E3779B9u;
+        rk[2 * r + 1] = k1 + (uint32_t)r * 0xBB67AE85u;
     }
-    const WEval ev = warp_batch<UNIF>(sv, sh.tab, sh.sig, sh.act, K, lo, hi, vmask, sc.pid, k0, k1, lane);
-    const uint32_t lq = ql == 0 ? lo[0] : ql == 1 ? lo[1] : ql == 2 ? lo[2] : lo[3];
-    const uint32_t hq = ql == 0 ? hi[0] : ql == 1 ? hi[1] : ql == 2 ? hi[2] : hi[3];
+    WHeads heads;
+    heads.make((uint32_t)(idx[b0] >> 32), sc.pid, rk, lane);
+    const WEval ev = warp_batch<UNIF>(
+        sv, sh.tw, sh.sig, sh.act, K, [&](int q) { return idx[b0 + q]; }, vmask, heads, sc.pid, rk, lane);
+    const unsigned long long iq = idx[b0 + ql < n ? b0 + ql : n - 1];
+    const uint32_t lq = (uint32_t)iq, hq = (uint32_t)(iq >> 32);
     const uint32_t wa = accept_word(lq, hq, sc.pid, K, k0, k1);
     const Fast f = warp_eval<UNIF>(ev, sc, wa);
     const bool valid = lane < kWQ && ((vmask >> lane) & 1u);
-    const bool slow = fabsf(f.d) < f.guard || min(ev.wmin, wa) < kTailBucket;
+    const bool slow = fabsf(f.d) < f.guard || ev.tail || wa < kTailBucket;
     const size_t rowlen = 8 + 2 * (size_t)K;
     if (valid && !slow) {
         double *row = out + (b0 + lane) * rowlen;
@@ -650,7 +761,7 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
             ((unsigned long long)__shfl_sync(0xffffffffu, hq, q) << 32) | __shfl_sync(0xffffffffu, lq, q);
         Out64 o;
         double inv;
-        eval64_warp<UNIF>(P, id, k0, k1, s_x[warp], lane, o, inv);
+        eval64_warp<UNIF>(P, id, k0, k1, sx, lane, o, inv);
         double *row = out + (b0 + q) * rowlen;
         if (lane == 0) {
             row[0] = o.delta;
@@ -663,7 +774,7 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
             row[7] = o.S;
         }
         for (int m = lane; m < K; m += 32) {
-            const double2 v = s_x[warp][m];
+            const double2 v = sx[m];
             row[8 + m] = (float)(v.x * inv);
             row[8 + K + m] = (float)(v.y * inv);
         }
@@ -675,7 +786,7 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
         const float inv = __shfl_sync(0xffffffffu, f.inv, q);
         double *row = out + (b0 + q) * rowlen;
         for (int m = lane; m < K; m += 32) {
-            const float2 v = sv[q * kWS + wpos(m)];
+            const float2 v = sv[q * kWS + m];
             row[8 + m] = v.x * inv;
             row[8 + K + m] = v.y * inv;
         }
@@ -698,7 +809,7 @@ void triad_kernels_k128(TriadKernels *t) {
     t->replay[0] = (const void *)k_replay_warp<false>;
     t->replay[1] = (const void *)k_replay_warp<true>;
     t->replay_per_block = 32 * kReplayWarps / 32 * kWQ;
-    t->xfer_bytes_per_thread = 0;
+    t->xfer_bytes_per_thread = kWarpWords * (int)sizeof(float2) / 32;  // the warps' slabs
     t->n_variants = 3;
 }
 
