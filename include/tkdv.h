@@ -244,6 +244,18 @@ int sampler_samples(tkdv_sampler *h, void *dst, int dst_on_device, uint64_t max_
    record of device memory for the call.  Errors: INVALID_ARG, OOM, CUDA. */
 int sampler_field_maxima(tkdv_sampler *h, uint64_t max_records, double *umax, int32_t *jmax, uint64_t *n_out);
 
+/* sampler_extreme_field: the 1-in-m event of `point` (Figs. 8-11): among the m
+   accepted fields with the smallest proposal index, of the first
+   min(max_records, kept) records, the one with the largest displacement on
+   the 2K-point grid (sampler_field_maxima).  *idx, *umax, *jmax and xhat (2K
+   floats, [cosine | sine]) describe it; all are host pointers.  *n_found
+   receives the number of fields of the point among those records; when it is
+   below m (m >= 1) nothing else is written.  Runs on the handle's stream
+   (synchronises) in the handle's buffers; allocates device memory for the
+   call only above 4M records.  Errors: INVALID_ARG, OOM, CUDA. */
+int sampler_extreme_field(tkdv_sampler *h, int point, uint64_t m, uint64_t max_records, uint64_t *idx, double *umax,
+                          int32_t *jmax, float *xhat, uint64_t *n_found);
+
 /* sampler_reset: zero statistics, the record ring and the running indices. */
 int sampler_reset(tkdv_sampler *h);
 

@@ -38,7 +38,7 @@ EXPORTED = ["tkdv_record_bytes", "sampler_create", "sampler_create_ex", "sampler
             "sampler_replay", "sampler_autotune", "sampler_launch_config", "sampler_last_error",
             "sampler_destroy", "tkdv_alpha_star", "tkdv_log_M", "sampler_run_static",
             "sampler_set_trace", "tkdv_check_radius_error", "tkdv_check_radius_error_log",
-            "sampler_h3_form", "sampler_batch_run", "sampler_set_launch", "tkdv_mlp_create", "tkdv_mlp_destroy", "tkdv_mlp_last_error",
+            "sampler_h3_form", "sampler_batch_run", "sampler_set_launch", "sampler_extreme_field", "tkdv_mlp_create", "tkdv_mlp_destroy", "tkdv_mlp_last_error",
             "tkdv_mlp_features", "tkdv_mlp_get_params", "tkdv_mlp_set_params", "tkdv_mlp_infer",
             "tkdv_mlp_set_data", "tkdv_mlp_set_data_records", "tkdv_mlp_rows", "tkdv_mlp_step"]
 MLP_NPARAM = 8640
@@ -134,6 +134,7 @@ def lib():
             L.tkdv_check_radius_error.argtypes = [dp, C.POINTER(C.c_uint32)]
             L.tkdv_check_radius_error_log.argtypes = [dp, C.POINTER(C.c_uint32)]
             L.sampler_field_maxima.argtypes = [vp, u64, dp, C.POINTER(C.c_int32), u64p]
+            L.sampler_extreme_field.argtypes = [vp, i, u64, u64, u64p, dp, C.POINTER(C.c_int32), fp, u64p]
             L.sampler_run_static.argtypes = [i, C.POINTER(tkdv_point), u64, u64, u64, vp, u64, u64p,
                                              C.POINTER(tkdv_stats), vp]
             _lib = L
@@ -159,6 +160,16 @@ def sampler_field_maxima(h, max_records):
     _check(lib().sampler_field_maxima(h, max_records, _dptr(umax), jm.ctypes.data_as(C.POINTER(C.c_int32)),
                                       C.byref(n)), h)
     return umax[:n.value], jm[:n.value]
+
+
+def sampler_extreme_field(h, K, point, m, max_records):
+    """(number of fields of the point, (idx, umax, j, xhat) of the extreme one
+    among its first m, or None when there are fewer)."""
+    idx, umax, jm, n = C.c_uint64(), C.c_double(), C.c_int32(), C.c_uint64()
+    xhat = np.zeros(2 * K, dtype=np.float32)
+    _check(lib().sampler_extreme_field(h, point, m, max_records, C.byref(idx), C.byref(umax), C.byref(jm),
+                                       _fptr(xhat), C.byref(n)), h)
+    return int(n.value), (idx.value, umax.value, jm.value, xhat) if n.value >= m else None
 
 
 def tkdv_check_radius_error():
@@ -593,15 +604,16 @@ class Sampler:
         of `point` (by proposal index) the one with the largest displacement
         on the 2K-point grid.  Returns a dict (idx, umax, xi, xhat) or None
         when fewer than m fields were kept."""
-        rec = self.samples(max_records)
-        umax, jm = self.field_maxima(max_records)
-        sel = np.nonzero(rec["point"] == point)[0]
-        if len(sel) < m:
+        if m < 0:  # all but the last -m
+            m = max(0, sampler_extreme_field(self.h, self.K, point, 1 << 62, max_records)[0] + m)
+        if m == 0:
+            raise ValueError("the extreme of no fields")
+        _, best = sampler_extreme_field(self.h, self.K, point, m, max_records)
+        if best is None:
             return None
-        sel = sel[np.argsort(rec["idx"][sel], kind="stable")[:m]]
-        b = sel[int(np.argmax(umax[sel]))]
-        return {"idx": int(rec["idx"][b]), "umax": float(umax[b]),
-                "xi": float(-np.pi + np.pi * jm[b] / self.K), "xhat": rec["xhat"][b].astype(np.float64)}
+        idx, umax, j, xhat = best
+        return {"idx": int(idx), "umax": float(umax), "xi": float(-np.pi + np.pi * j / self.K),
+                "xhat": xhat.astype(np.float64)}
 
     def replay(self, p, idx, seed):
         return sampler_replay(self.h, p, self.K, idx, seed)

@@ -854,6 +854,55 @@ int sampler_field_maxima(tkdv_sampler *h, uint64_t max_records, double *umax, in
     return TKDV_OK;
 }
 
+int sampler_extreme_field(tkdv_sampler *h, int point, uint64_t m, uint64_t max_records, uint64_t *idx, double *umax,
+                          int32_t *jmax, float *xhat, uint64_t *n_found) {
+    if (!h || m == 0 || !idx || !umax || !jmax || !xhat || !n_found) return TKDV_ERR_INVALID_ARG;
+    CK(cudaStreamSynchronize(h->stream));
+    unsigned long long cnt = 0;
+    CK(cudaMemcpy(&cnt, h->d_ring_count, 8, cudaMemcpyDeviceToHost));
+    unsigned long long n = std::min<unsigned long long>(cnt, h->dev.ring_cap);
+    n = std::min<unsigned long long>(n, max_records);
+    *n_found = 0;
+    if (!n || point < 0 || point >= h->n_points) return TKDV_OK;
+    // the FP64 queue is free between runs; a larger ring gets its own scratch
+    const unsigned long long mm = std::min<unsigned long long>(m, n);
+    const size_t need = extreme_scratch_bytes(n, mm);
+    void *scratch = h->d_refine, *own = nullptr;
+    if (need > sizeof(RefineItem) * (size_t)kRefineCap) {
+        if (cudaMalloc(&own, need) != cudaSuccess) return fail(h, TKDV_ERR_OOM, "extreme field: out of device memory");
+        scratch = own;
+    }
+    ExtremeBufs b{};
+    unsigned long long found = 0, best_idx = 0, best_slot = 0;
+    cudaError_t e = launch_extreme((const unsigned char *)h->d_ring, h->rec_bytes, n, h->K, (const PointConst *)h->d_pts,
+                                   (uint32_t)point, mm, scratch, &b, h->stream);
+    std::vector<unsigned char> out(24 * mm);  // slot, idx, umax, jmax
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out.data(), b.slot, 24 * mm, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&found, b.n_match, 8, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess && found >= m) {
+        const unsigned long long *slot = (const unsigned long long *)out.data(), *id = slot + mm;
+        const float *u = (const float *)(id + mm);
+        const int *j = (const int *)(u + mm);
+        size_t best = 0;
+        for (size_t i = 1; i < mm; ++i)  // the first of the largest, by index, then by ring position
+            if (u[i] > u[best] ||
+                (u[i] == u[best] && (id[i] < id[best] || (id[i] == id[best] && slot[i] < slot[best]))))
+                best = i;
+        best_idx = id[best];
+        best_slot = slot[best];
+        *umax = u[best];
+        *jmax = j[best];
+        e = cudaMemcpy(xhat, (const unsigned char *)h->d_ring + best_slot * h->rec_bytes + 32, 8 * (size_t)h->K,
+                       cudaMemcpyDeviceToHost);
+        *idx = best_idx;
+    }
+    if (own) cudaFree(own);
+    if (e != cudaSuccess) return fail(h, TKDV_ERR_CUDA, cudaGetErrorString(e));
+    *n_found = found;
+    return TKDV_OK;
+}
+
 int sampler_reset(tkdv_sampler *h) {
     if (!h) return TKDV_ERR_INVALID_ARG;
     CK(cudaStreamSynchronize(h->stream));

@@ -206,5 +206,17 @@ void fill_point_const(int K, const tkdv_point &q, const double *s2, double logM,
 // Largest displacement of n kept records on the 2K-point grid (fields.cu).
 cudaError_t launch_field_max(const unsigned char *ring, unsigned long long rec_bytes, unsigned long long n, int K,
                              const PointConst *pts, float *umax, int *jmax, cudaStream_t st);
+// The m records of `point` with the smallest (index, ring position) among the
+// first n (n, m >= 1) and their largest displacements, in any order, into
+// scratch (extreme_scratch_bytes); valid where *n_match >= m.
+struct ExtremeBufs {
+    unsigned long long *n_match, *slot, *idx;
+    float *umax;
+    int *jmax;
+};
+size_t extreme_scratch_bytes(unsigned long long n, unsigned long long m);
+cudaError_t launch_extreme(const unsigned char *ring, unsigned long long rec_bytes, unsigned long long n, int K,
+                           const PointConst *pts, uint32_t point, unsigned long long m, void *scratch,
+                           ExtremeBufs *out, cudaStream_t st);
 
 }  // namespace tkdv
