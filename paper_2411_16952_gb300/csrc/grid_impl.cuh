@@ -228,6 +228,7 @@ struct GridWG {
     // mode_consts of the point by pairs of modes (2j, 2j + 1) = Philox block
     // j: (s, s', s^2, s'^2) and ((m+1)^2 s^2, (m+2)^2 s'^2, act, act')
     float4 mp[KMAX / 2][2];
+    PhiloxHead heads[KMAX / 2 + 1];  // blocks 0..KMAX/2-1 and the accept word's
 };
 
 // One row of a tile between its draw and its decision.
@@ -243,7 +244,10 @@ struct GridRow {
 // (A second A tile per warpgroup, drawing tile t+1 before waiting for the
 // products of tile t, measured 8 % slower at three warpgroups than one tile
 // with the product-free decision terms made before the wait.)
-template <int KMAX, bool UNIF, int NWG, int UNR>
+// HEADS: see k_sample_triad; here with three and four warpgroups (32 modes 12.93
+// -> 13.00e9 and 12.11 -> 12.19e9, 16 modes 21.1 -> 21.8e9 proposals/s; with two
+// warpgroups 10.71 -> 10.40e9, and 5.61 -> 5.08e9 at 64 modes).
+template <int KMAX, bool UNIF, int NWG, int UNR, bool HEADS = (NWG >= 3)>
 __global__ void __launch_bounds__(128 * NWG, 1)
     k_sample_grid(const __grid_constant__ DevBufs B, const __grid_constant__ RunArgs A, uint32_t k0, uint32_t k1,
                   const unsigned char *__restrict__ bimg, int gridN) {
@@ -343,11 +347,9 @@ __global__ void __launch_bounds__(128 * NWG, 1)
             W.mp[t][1] = make_float4(a.z, b.z, a.w, b.w);
         }
         const Scal sc = load_scal(P);
-        wg_sync(g);
         float maxd = -INFINITY;
         uint32_t nacc = 0;  // accepted draws of this warp in this chunk (the same in every lane)
 
-        const uint32_t n_tiles = (n_here + 127u) / 128u;
         // ---- 3./4. the products and the decision of one row
         auto consume = [&](const GridRow &r) {
             const unsigned long long idx = r.idx;
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(128 * NWG, 1)
             const float S = Sraw * inv2;
             const float tS = sc.cS * S;
             const float tQ = UNIF ? 0.f : sc.cQ * logf(zz * inv2);
-            const uint32_t wa = PhiloxRow(lo, hi, sc.pid, A.rk.k).block((uint32_t)((sc.K + 1) / 2)).x;
+            const uint32_t wa = PhiloxOf<HEADS>(lo, hi, sc.pid, A.rk.k, W.heads).block((uint32_t)((sc.K + 1) / 2)).x;
             const float lnU = -0.5f * rho_fast(wa);
             // ---- 3. wait for the products, sum 2 C (C^2 + 3 S^2) of this row
             float cube = 0.f;
@@ -459,10 +461,21 @@ __global__ void __launch_bounds__(128 * NWG, 1)
                 nacc += (uint32_t)__popc(ma);
             }
         };
+        // with heads the chunk in one part, or in two where its indices cross a
+        // multiple of 2^32 (the heads hold for one upper half)
+        for (uint32_t i1 = 0, end = n_here; i1 < n_here; i1 = end) {
+        if constexpr (HEADS) {
+            end = i1 + (uint32_t)umin64(n_here - i1, 0x100000000ull - (uint32_t)(cbase + i1));
+            if (i1) wg_sync(g);  // the first part's readers of the heads are done
+            if (t <= KMAX / 2)
+                W.heads[t] = philox_head((uint32_t)t, (uint32_t)((cbase + i1) >> 32), sc.pid, A.rk.k);
+        }
+        wg_sync(g);
+        const uint32_t n_tiles = (end - i1 + 127u) / 128u;
         for (uint32_t trip = 0; trip < n_tiles; ++trip) {
             GridRow cur;
             {  // ---- 1. this thread's row of the tile
-                const uint32_t i = trip * 128u + (uint32_t)t;
+                const uint32_t i = i1 + trip * 128u + (uint32_t)t;
                 const unsigned long long idx = cbase + i;
                 const uint32_t lo = (uint32_t)idx, hi = (uint32_t)(idx >> 32);
                 // ---- 1. the row of X: eight modes (four Philox blocks) at a time,
@@ -470,7 +483,7 @@ __global__ void __launch_bounds__(128 * NWG, 1)
                 // the mode sums over even and odd modes in packed pairs
                 f32x2_t nrm2p = 0ull, Srawp = 0ull, zzp = 0ull, esump = 0ull;
                 uint32_t wmin = 0xFFFFFFFFu;
-                const PhiloxRow prow(lo, hi, sc.pid, A.rk.k);
+                const PhiloxOf<HEADS> prow(lo, hi, sc.pid, A.rk.k, W.heads);
 #pragma unroll(UNR)
                 for (int c8 = 0; c8 < KMAX / 8; ++c8) {
                     float vx[8], vy[8];
@@ -502,7 +515,7 @@ __global__ void __launch_bounds__(128 * NWG, 1)
                 }
                 float e0, e1;
                 cur.idx = idx;
-                cur.valid = i < n_here;
+                cur.valid = i < end;
                 upk2(nrm2p, e0, e1);
                 cur.nrm2 = e0 + e1;
                 upk2(Srawp, e0, e1);
@@ -542,6 +555,7 @@ __global__ void __launch_bounds__(128 * NWG, 1)
                 }
             }
             consume(cur);
+        }
         }
 
         // ---- outputs of this warp's accepted draws of the chunk, 32 at a time:

@@ -75,7 +75,7 @@ struct PhiloxRow {
 // gives four words per (j, hi, pid, key) (PhiloxHead), and what does not depend
 // on j one product per proposal (PhiloxTail), so a block takes 15 wide products
 // and 17 xors instead of 20 and 20.
-struct PhiloxHead {
+struct __align__(16) PhiloxHead {
     uint32_t a, b, c, d;
 };
 __device__ __forceinline__ PhiloxHead philox_head(uint32_t j, uint32_t hi, uint32_t pid, const uint32_t *rk) {
@@ -107,6 +107,18 @@ struct PhiloxTail {
                            (uint32_t)(p0 >> 32) ^ c.w ^ rk[2 * r + 1], (uint32_t)p0);
         }
         return c;
+    }
+};
+
+// The blocks of one proposal from a table of heads (heads[j] for block j).
+struct PhiloxTable {
+    PhiloxTail tail;
+    const PhiloxHead *heads;
+    __device__ __forceinline__ PhiloxTable(uint32_t lo, uint32_t hi, const uint32_t *rk, const PhiloxHead *h)
+        : tail(lo, hi, rk), heads(h) {}
+    __device__ __forceinline__ uint4 block(uint32_t j) const {
+        const uint4 h = *reinterpret_cast<const uint4 *>(heads + j);
+        return tail.block(PhiloxHead{h.x, h.y, h.z, h.w});
     }
 };
 
@@ -241,6 +253,8 @@ __device__ __forceinline__ uint32_t fkey(float f) {
     uint32_t b = __float_as_uint(f);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
+
+__device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -713,7 +727,28 @@ __host__ __device__ constexpr int xfer_stride() { return 2 * KMAX + 4; }
 // tallies its spectrum and writes its record itself.  The first pays off
 // once a warp iteration often holds an accepted draw, the second can spill
 // less under a tight register budget; the autotune times both.
-template <int KMAX, bool UNIF, int NT, int MINB, bool SIR = false, bool XFER = true>
+// HEADS: the Philox blocks from the chunk's table of heads (PhiloxTable), else
+// from the counter (PhiloxRow).  The table saves a sixth of the rounds but
+// puts a shared-memory load in front of every block, which pays off where four
+// warps per scheduler hide it (the variants held to 128 registers, from 16
+// modes on: triad 10.00 -> 10.39 and 9.99 -> 10.58, 16 modes 22.46 -> 22.72e9
+// proposals/s) and not with fewer (8 modes 36.0 -> 24.7, 64 modes at 128 threads
+// 3.47 -> 3.02).
+template <bool HEADS>
+struct PhiloxOf;
+template <>
+struct PhiloxOf<true> : PhiloxTable {
+    __device__ __forceinline__ PhiloxOf(uint32_t lo, uint32_t hi, uint32_t, const uint32_t *rk, const PhiloxHead *h)
+        : PhiloxTable(lo, hi, rk, h) {}
+};
+template <>
+struct PhiloxOf<false> : PhiloxRow {
+    __device__ __forceinline__ PhiloxOf(uint32_t lo, uint32_t hi, uint32_t pid, const uint32_t *rk, const PhiloxHead *)
+        : PhiloxRow(lo, hi, pid, rk) {}
+};
+
+template <int KMAX, bool UNIF, int NT, int MINB, bool SIR = false, bool XFER = true,
+          bool HEADS = (KMAX >= 16 && MINB == 2)>
 __global__ void __launch_bounds__(NT, MINB)
     k_sample_triad(const __grid_constant__ DevBufs B, const __grid_constant__ RunArgs A, uint32_t k0, uint32_t k1) {
     __shared__ uint32_t s_hist[kHistBins];
@@ -726,6 +761,7 @@ __global__ void __launch_bounds__(NT, MINB)
     __shared__ uint32_t s_chunk;
     __shared__ float s_sig[KMAX], s_act[KMAX];
     __shared__ float4 s_md[KMAX];
+    __shared__ PhiloxHead s_heads[HEADS ? KMAX / 2 + 1 : 1];  // blocks 0..KMAX/2-1 and the accept word's
     // dynamic: per thread, its accepted draw's scaled state (x | y), padded
     // (kXferStride floats apart, so that the lanes' vector stores spread over
     // the banks); absent in the SIR form
@@ -770,17 +806,26 @@ __global__ void __launch_bounds__(NT, MINB)
             s_md[tid] = mode_consts<UNIF>(sg, ac, tid);
         }
         const Scal sc = load_scal(P);
-        __syncthreads();
 
         float maxd = -INFINITY;
         float a_sir[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // SIR: w, w^2, w S, w u0^p
-        for (uint32_t i0 = 0; i0 < n_here; i0 += NT) {
+        // with heads the chunk in one part, or in two where its indices cross a
+        // multiple of 2^32 (the heads hold for one upper half)
+        for (uint32_t i1 = 0, end = n_here; i1 < n_here; i1 = end) {
+        if constexpr (HEADS) {
+            end = i1 + (uint32_t)umin64(n_here - i1, 0x100000000ull - (uint32_t)(base + i1));
+            if (i1) __syncthreads();  // the first part's readers of the heads are done
+            if (tid <= KMAX / 2)
+                s_heads[tid] = philox_head((uint32_t)tid, (uint32_t)((base + i1) >> 32), sc.pid, A.rk.k);
+        }
+        __syncthreads();
+        for (uint32_t i0 = i1; i0 < end; i0 += NT) {
             const uint32_t i = i0 + (uint32_t)tid;
-            const bool valid = i < n_here;
+            const bool valid = i < end;
             const unsigned long long idx = base + i;
             const uint32_t lo = (uint32_t)idx, hi = (uint32_t)(idx >> 32);
             Draw<KMAX> dr;
-            const PhiloxRow prow(lo, hi, sc.pid, A.rk.k);
+            const PhiloxOf<HEADS> prow(lo, hi, sc.pid, A.rk.k, s_heads);
             // the per-mode constants from the table, or formed from sigma and
             // act where the table's loads spill under the hand-off variant's
             // register budget (the same values either way)
@@ -948,6 +993,7 @@ __global__ void __launch_bounds__(NT, MINB)
                     }
                 }
             }
+        }
         }
 
         // chunk done: flush this CTA's partials into the point's StatBlock

@@ -183,6 +183,13 @@ void build_grid_image(int K, int kmax, int ka, int N, unsigned char *out);
 
 constexpr int kTriadVariantThreads[6] = {128, 256, 256, 128, 256, 256};
 
+// The triad form's launch variant where the caller leaves it open: two
+// 256-thread CTAs per SM from 9 to 32 modes (held to 128 registers; 23.0
+// against 18.6e9 proposals/s for one CTA at 16 modes, 10.4 against 9.6e9 at 32)
+// and for the warp form; one CTA of 256 below (no difference at 8) and above
+// (3.0 and 1.8e9 against 2.6 and 2.6e9 at 64 and 40 modes).
+inline int default_triad_variant(int kmax) { return kmax == 16 || kmax == 32 || kmax == 128 ? 2 : 1; }
+
 inline size_t record_bytes(int K) {
     size_t b = 32 + 8 * (size_t)K;
     return (b + 15) & ~(size_t)15;
