@@ -1075,11 +1075,12 @@ static __device__ double poisson_tail_d(double lambda, int k) {
 constexpr int kMaxCopies = (1 << 24) - 1;  // copies fit the record's 24-bit field
 
 // ---- FP64 decision of the guard-band proposals ---------------------------
-// A warp takes up to 32 queued proposals.  The K modes of a proposal and its
-// triads are spread over a segment of kLanes lanes (32 / kLanes proposals at
-// a time), their sums meet in the segment by shuffles, and lane q keeps those
-// of proposal q; the scalar part of the decision (1/|x|, the logarithms, the
-// SIR copy number) then runs once for the whole batch, a proposal per lane.
+// A CTA takes up to 32 queued proposals.  The K modes of a proposal and its
+// triads are spread over a segment of kLanes lanes of a warp (32 / kLanes
+// proposals at a time, the four warps in turn), and their sums meet in the
+// segment by shuffles; the scalar part of the decision (1/|x|, the logarithms,
+// the SIR copy number) then runs once for the whole batch, a proposal per lane
+// of the first warp.
 //
 // What bounds it: an FP64 instruction of a warp holds its scheduler for 64
 // cycles (measured, dependent or not, whatever the number of active lanes).
@@ -1098,7 +1099,7 @@ struct RefineShape {
     static constexpr int kModes = KMAX / kLanes > 1 ? KMAX / kLanes : 1;  // modes of one lane
     static constexpr int kBatch = 32;
     static constexpr int kWarps = 4;
-    static constexpr size_t kSmem = sizeof(double2) * kWarps * kBatch * KMAX;
+    static constexpr size_t kSmem = sizeof(double2) * kBatch * KMAX;
 };
 
 // Sums over a segment's lanes, the same values in every lane of it.
@@ -1114,21 +1115,21 @@ __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t
     using RS = RefineShape<KMAX>;
     constexpr int LANES = RS::kLanes, GROUP = RS::kGroup, MODES = RS::kModes;
     extern __shared__ __align__(16) unsigned char s_refine[];
+    __shared__ double s_sum[RS::kBatch][5];  // |x|^2, S|x|^2, Q|x|^2, u(0)|x|/u0s, T|x|^3
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = lane / LANES, l = lane % LANES;
-    double2 *slab = reinterpret_cast<double2 *>(s_refine) + (size_t)warp * RS::kBatch * KMAX;
+    double2 *slab = reinterpret_cast<double2 *>(s_refine);
     const uint32_t n = min(*(volatile uint32_t *)&B.counters[1], B.refine_cap);
-    // batches of consecutive items, first to distinct CTAs, then to the warps
-    // of a CTA (one per scheduler), as small as the warps allow
-    const uint32_t nw = gridDim.x * RS::kWarps;
-    uint32_t batch = (n + nw - 1) / nw;
-    batch = min((batch + GROUP - 1) / GROUP * GROUP, (uint32_t)RS::kBatch);
-    for (uint32_t first = ((uint32_t)warp * gridDim.x + blockIdx.x) * batch; first < n; first += nw * batch) {
+    // batches of consecutive items, as small as the CTAs allow; full ones where
+    // an SIR run has more of them than the ring has room for, so that the
+    // records that do fit stay runs of consecutive items
+    uint32_t batch = min((n + gridDim.x - 1) / gridDim.x, (uint32_t)RS::kBatch);
+    if (B.sir && n > B.ring_cap) batch = RS::kBatch;
+    for (uint32_t first = blockIdx.x * batch; first < n; first += gridDim.x * batch) {
         const uint32_t cnt = min(batch, n - first);
-        double nrm2 = 1.0, Sraw = 0.0, zz = 1.0, u0raw = 0.0, T = 0.0;  // of item first + lane
-        __syncwarp();  // the slab's readers of the previous batch are done
+        __syncthreads();  // the slab's readers of the previous batch are done
 #pragma unroll 1
-        for (uint32_t g0 = 0; g0 < cnt; g0 += GROUP) {
+        for (uint32_t g0 = (uint32_t)warp * GROUP; g0 < cnt; g0 += RS::kWarps * GROUP) {
             const uint32_t q = min(g0 + (uint32_t)sub, cnt - 1);  // (an idle segment repeats the last item)
             const RefineItem it = B.refine[first + q];
             const PointConst *P = B.pts + it.point;
@@ -1180,21 +1181,21 @@ __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t
             az = seg_sum<LANES>(az);
             au = seg_sum<LANES>(au);
             at = seg_sum<LANES>(at);
-            // lane g0 + s takes the sums of segment s
-            const int src = ((lane - (int)g0) & (GROUP - 1)) * LANES;
-            const double on = __shfl_sync(0xffffffffu, an, src), oS = __shfl_sync(0xffffffffu, aS, src),
-                         oz = __shfl_sync(0xffffffffu, az, src), ou = __shfl_sync(0xffffffffu, au, src),
-                         ot = __shfl_sync(0xffffffffu, at, src);
-            if (lane >= (int)g0 && lane < (int)g0 + GROUP) {
-                nrm2 = on;
-                Sraw = oS;
-                zz = oz;
-                u0raw = ou;
-                T = ot;
+            if (l == 0) {
+                double *d = s_sum[g0 + (uint32_t)sub];
+                d[0] = an;
+                d[1] = aS;
+                d[2] = az;
+                d[3] = au;
+                d[4] = at;
             }
         }
+        __syncthreads();
+        if (warp > 0) continue;
         // the decision of item first + lane (the formulas of eval64)
         const bool valid = (uint32_t)lane < cnt;
+        const double *sums = s_sum[min((uint32_t)lane, cnt - 1)];
+        const double nrm2 = sums[0], Sraw = sums[1], zz = sums[2], u0raw = sums[3], T = sums[4];
         const RefineItem it = B.refine[first + min((uint32_t)lane, cnt - 1)];
         const PointConst *P = B.pts + it.point;
         StatBlock *st = B.stats + it.point;
