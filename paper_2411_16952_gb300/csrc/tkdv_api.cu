@@ -415,9 +415,17 @@ int run_ranges(tkdv_sampler *h, const unsigned long long *idx0, const unsigned l
     return enqueue(h);
 }
 
-int check_status(tkdv_sampler *h) {
-    uint32_t st = 0;
-    CK(cudaMemcpy(&st, h->d_status, 4, cudaMemcpyDeviceToHost));
+// Bytes from the statistics to the end of the run state: one allocation holds
+// them, the record count, the status word and the run counters, so that a
+// reset is one memset and reading the statistics one copy.
+struct StateTail {
+    unsigned long long ring_count;
+    uint32_t status, pad;
+    uint32_t counters[4];
+};
+size_t state_bytes(const tkdv_sampler *h) { return sizeof(StatBlock) * (size_t)h->n_points + sizeof(StateTail); }
+
+int check_status(tkdv_sampler *h, uint32_t st) {
     if (st) CK(cudaMemset(h->d_status, 0, 4));
     if (st & (kStatusDeadline | kStatusMbarTimeout))
         return fail(h, TKDV_ERR_TIMEOUT,
@@ -430,8 +438,7 @@ int check_status(tkdv_sampler *h) {
 void free_all(tkdv_sampler *h) {
     if (h->exec) cudaGraphExecDestroy(h->exec);
     if (h->graph) cudaGraphDestroy(h->graph);
-    for (void *p : {h->d_pts, h->d_stats, h->d_ring, h->d_ring_count, h->d_refine, h->d_counters, h->d_status,
-                    h->d_bimg, h->d_accs})
+    for (void *p : {h->d_pts, h->d_stats, h->d_ring, h->d_refine, h->d_bimg, h->d_accs})
         if (p) cudaFree(p);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
@@ -634,12 +641,15 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
     };
     int rc;
     if ((rc = alloc(&h->d_pts, sizeof(PointConst) * n_points))) return bail(rc);
-    if ((rc = alloc(&h->d_stats, sizeof(StatBlock) * n_points))) return bail(rc);
+    if ((rc = alloc(&h->d_stats, state_bytes(h)))) return bail(rc);
+    {
+        StateTail *t = (StateTail *)((StatBlock *)h->d_stats + n_points);
+        h->d_ring_count = &t->ring_count;
+        h->d_status = &t->status;
+        h->d_counters = t->counters;
+    }
     if ((rc = alloc(&h->d_ring, h->rec_bytes * cap))) return bail(rc);
-    if ((rc = alloc(&h->d_ring_count, 8))) return bail(rc);
     if ((rc = alloc(&h->d_refine, sizeof(RefineItem) * (size_t)kRefineCap))) return bail(rc);
-    if ((rc = alloc(&h->d_counters, 16))) return bail(rc);
-    if ((rc = alloc(&h->d_status, 4))) return bail(rc);
     if (opt->cuda_stream) {
         h->stream = (cudaStream_t)opt->cuda_stream;
     } else {
@@ -663,10 +673,7 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
     }
     h->pc = h->launch.form == TKDV_H3_GRID_BF16X3 ? h->pc_grid : h->pc_triad;
     e = cudaMemcpy(h->d_pts, h->pc.data(), sizeof(PointConst) * n_points, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(h->d_stats, 0, sizeof(StatBlock) * n_points);
-    if (e == cudaSuccess) e = cudaMemset(h->d_ring_count, 0, 8);
-    if (e == cudaSuccess) e = cudaMemset(h->d_counters, 0, 16);
-    if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, 4);
+    if (e == cudaSuccess) e = cudaMemset(h->d_stats, 0, state_bytes(h));
     if (e != cudaSuccess) {
         h->err = std::string("initialising device buffers: ") + cudaGetErrorString(e);
         return bail(TKDV_ERR_CUDA);
@@ -731,7 +738,9 @@ int sampler_run_ranges(tkdv_sampler *h, const uint64_t *idx0, const uint64_t *co
 int sampler_sync(tkdv_sampler *h) {
     if (!h) return TKDV_ERR_INVALID_ARG;
     CK(cudaStreamSynchronize(h->stream));
-    return check_status(h);
+    uint32_t st = 0;
+    CK(cudaMemcpy(&st, h->d_status, 4, cudaMemcpyDeviceToHost));
+    return check_status(h, st);
 }
 
 int sampler_set_trace(tkdv_sampler *h, void *dev_buf, uint64_t n) {
@@ -750,9 +759,11 @@ int sampler_set_deadline_ns(tkdv_sampler *h, uint64_t ns) {
 
 int sampler_stats(tkdv_sampler *h, tkdv_stats *out, int n_out) {
     if (!h || !out || n_out < 0 || n_out > h->n_points) return TKDV_ERR_INVALID_ARG;
-    int rc = sampler_sync(h);
-    std::vector<StatBlock> sb(h->n_points);
-    CK(cudaMemcpy(sb.data(), h->d_stats, sizeof(StatBlock) * h->n_points, cudaMemcpyDeviceToHost));
+    CK(cudaStreamSynchronize(h->stream));
+    std::vector<unsigned char> state(state_bytes(h));
+    CK(cudaMemcpy(state.data(), h->d_stats, state.size(), cudaMemcpyDeviceToHost));
+    const StatBlock *sb = (const StatBlock *)state.data();
+    const int rc = check_status(h, ((const StateTail *)(sb + h->n_points))->status);
     for (int p = 0; p < n_out; ++p) {
         const StatBlock &s = sb[p];
         tkdv_stats &o = out[p];
@@ -906,9 +917,7 @@ int sampler_extreme_field(tkdv_sampler *h, int point, uint64_t m, uint64_t max_r
 int sampler_reset(tkdv_sampler *h) {
     if (!h) return TKDV_ERR_INVALID_ARG;
     CK(cudaStreamSynchronize(h->stream));
-    CK(cudaMemset(h->d_stats, 0, sizeof(StatBlock) * h->n_points));
-    CK(cudaMemset(h->d_ring_count, 0, 8));
-    CK(cudaMemset(h->d_status, 0, 4));
+    CK(cudaMemset(h->d_stats, 0, state_bytes(h)));
     std::fill(h->next_idx.begin(), h->next_idx.end(), 0ull);
     return TKDV_OK;
 }

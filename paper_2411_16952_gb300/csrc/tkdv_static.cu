@@ -170,14 +170,14 @@ extern "C" int sampler_run_static(int K, const tkdv_point *point, uint64_t idx0,
         }
         if (e != cudaSuccess) return TKDV_ERR_CUDA;
     }
-    StatBlock sb;
-    unsigned long long ring_count = 0;
-    uint32_t status = 0;
-    e = cudaMemcpyAsync(&sb, &hdr->stats, sizeof(sb), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&ring_count, &hdr->ring_count, 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&status, &hdr->status, 4, cudaMemcpyDeviceToHost, st);
+    StaticHeader back;  // everything after the point table in one copy
+    e = cudaMemcpyAsync(&back.stats, &hdr->stats, sizeof(StaticHeader) - offsetof(StaticHeader, stats),
+                        cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return TKDV_ERR_CUDA;
+    const StatBlock &sb = back.stats;
+    const unsigned long long ring_count = back.ring_count;
+    const uint32_t status = back.status;
     if (n_records) *n_records = std::min<unsigned long long>(ring_count, B.ring_cap);
     if (stats) {
         tkdv_stats &o = *stats;
