@@ -170,7 +170,7 @@ __device__ __forceinline__ float angle_f(uint32_t w) {
 
 // The hardware approximations of PTX (lg2, rsqrt, sin, cos .approx) in their
 // flush-to-zero forms.  Every argument the sampler gives them (u in
-// [2^-24, 1), rho >= 2^-25, |x|^2 > 0, angles of magnitude >= 2 pi 2^-24) and
+// [2^-24, 1), rho >= 1.6e-8, |x|^2 > 0, angles of magnitude >= 2 pi 2^-24) and
 // every result is a normal float, where the flushing forms return the same
 // documented approximation without handling for subnormal operands.
 __device__ __forceinline__ float lg2_approx(float x) {
@@ -1074,6 +1074,32 @@ static __device__ double poisson_tail_d(double lambda, int k) {
 }
 constexpr int kMaxCopies = (1 << 24) - 1;  // copies fit the record's 24-bit field
 
+// SIR: n = #{k >= 1 : U < P(N >= k)}, N ~ Poisson(lam); near: U within 1e-6 (in
+// log) of the tail value that decided n.
+static __device__ int sir_copies(double lam, double u, double lnU, bool &near) {
+    int n = 0;
+    double tk = poisson_tail_d(lam, 1);
+    while (n < kMaxCopies && u < tk) {
+        ++n;
+        tk = poisson_tail_d(lam, n + 1);
+    }
+    const double tn = n > 0 ? poisson_tail_d(lam, n) : 1.0;
+    near = fabs(lnU - log(tk)) < 1e-6 || (n > 0 && fabs(lnU - log(tn)) < 1e-6);
+    return n;
+}
+
+// u(0) statistics of `copies` copies of one field, into its point's block.
+__device__ __forceinline__ void tally_copies(StatBlock *st, const PointConst *P, float u0, unsigned long long copies) {
+    const float u2 = u0 * u0;
+    atomicAdd(&st->n_acc, copies);
+    atomicAdd(&st->hist[hist_bin(u0, __ldg(&P->hist_a), __ldg(&P->hist_b))], copies);
+    atomicAdd(&st->exc[exc_bin(u0, __ldg(&P->exc_a))], copies);
+    atomicAdd(&st->q[0], copies * (unsigned long long)__float2ll_rn(u0 * kQ1));
+    atomicAdd(&st->q[1], copies * (unsigned long long)__float2ll_rn(u2 * kQ2));
+    atomicAdd(&st->q[2], copies * (unsigned long long)__float2ll_rn(u2 * u0 * kQ3));
+    atomicAdd(&st->q[3], copies * (unsigned long long)__float2ll_rn(u2 * u2 * kQ4));
+}
+
 // ---- FP64 decision of the guard-band proposals ---------------------------
 // A CTA takes up to 32 queued proposals.  The K modes of a proposal and its
 // triads are spread over a segment of kLanes lanes of a warp (32 / kLanes
@@ -1110,6 +1136,44 @@ __device__ __forceinline__ double seg_sum(double v) {
     return v;
 }
 
+// The FP64 pass of an SIR run that queues more draws than the ring has room
+// for, one proposal per thread.  The records that do not fit are counted per
+// point, and which points they fall on follows the order in which draws
+// finish: consecutive draws together, as in this form.
+template <int KMAX, bool UNIF>
+__device__ __noinline__ void refine_serial(const DevBufs &B, uint32_t n, uint32_t k0, uint32_t k1) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const RefineItem it = B.refine[i];
+        const PointConst *P = B.pts + it.point;
+        StatBlock *st = B.stats + it.point;
+        Out64 o;
+        float xh[2 * KMAX];
+        eval64<KMAX, UNIF>(P, it.idx, k0, k1, &o, xh);
+        atomicAdd(&st->n_refined, 1ull);
+        atomicMax(&st->maxd_key, (unsigned long long)fkey((float)o.delta));
+        bool near = false;
+        const unsigned long long copies = (unsigned long long)sir_copies(P->sir_c * exp(o.delta), o.u, o.lnU, near);
+        if (near) atomicAdd(&st->n_near, 1ull);
+        if (copies == 0) continue;
+        atomicAdd(&st->n_kept, 1ull);
+        tally_copies(st, P, o.u0, copies);
+        const int K = P->K;
+        for (int m = 0; m < K; ++m)
+            atomicAdd(&st->spec[m], copies * (unsigned long long)__float2ull_rn(
+                                                 fmaf(xh[m], xh[m], xh[K + m] * xh[K + m]) * kSpecScale));
+        const unsigned long long slot = atomicAdd(B.ring_count, 1ull);
+        if (slot < B.ring_cap) {
+            unsigned char *rec = B.ring + slot * B.rec_bytes;
+            write_header(rec, it.idx, it.point, 1u | (near ? 2u : 0u) | (uint32_t)copies << 8, o.H2, o.H3, o.u0,
+                         (float)o.delta);
+            float *f = reinterpret_cast<float *>(rec + 32);
+            for (int m = 0; m < 2 * K; ++m) f[m] = xh[m];
+        } else {
+            atomicAdd(&st->n_dropped, 1ull);
+        }
+    }
+}
+
 template <int KMAX, bool UNIF>
 __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t k1) {
     using RS = RefineShape<KMAX>;
@@ -1120,11 +1184,12 @@ __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t
     const int sub = lane / LANES, l = lane % LANES;
     double2 *slab = reinterpret_cast<double2 *>(s_refine);
     const uint32_t n = min(*(volatile uint32_t *)&B.counters[1], B.refine_cap);
-    // batches of consecutive items, as small as the CTAs allow; full ones where
-    // an SIR run has more of them than the ring has room for, so that the
-    // records that do fit stay runs of consecutive items
-    uint32_t batch = min((n + gridDim.x - 1) / gridDim.x, (uint32_t)RS::kBatch);
-    if (B.sir && n > B.ring_cap) batch = RS::kBatch;
+    if (B.sir && n > B.ring_cap) {
+        refine_serial<KMAX, UNIF>(B, n, k0, k1);
+        return;
+    }
+    // batches of consecutive items, as small as the CTAs allow
+    const uint32_t batch = min((n + gridDim.x - 1) / gridDim.x, (uint32_t)RS::kBatch);
     for (uint32_t first = blockIdx.x * batch; first < n; first += gridDim.x * batch) {
         const uint32_t cnt = min(batch, n - first);
         __syncthreads();  // the slab's readers of the previous batch are done
@@ -1219,19 +1284,8 @@ __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t
             atomicAdd(&st->n_refined, 1ull);
             atomicMax(&st->maxd_key, (unsigned long long)fkey((float)delta));
             if (B.sir) {
-                // SIR: n = #{k >= 1 : U < P(N >= k)}, N ~ Poisson(c exp(delta))
-                const double lam = P->sir_c * exp(delta);
-                int nc = 0;
-                double tk = poisson_tail_d(lam, 1);
-                while (nc < kMaxCopies && u < tk) {
-                    ++nc;
-                    tk = poisson_tail_d(lam, nc + 1);
-                }
-                // near: U within 1e-6 (in log) of the tail value that decided n
-                const double tn = nc > 0 ? poisson_tail_d(lam, nc) : 1.0;
-                near = fabs(lnU - log(tk)) < 1e-6 || (nc > 0 && fabs(lnU - log(tn)) < 1e-6);
-                if (nc > 0) atomicAdd(&st->n_kept, 1ull);
-                copies = (unsigned long long)nc;
+                copies = (unsigned long long)sir_copies(P->sir_c * exp(delta), u, lnU, near);
+                if (copies > 0) atomicAdd(&st->n_kept, 1ull);
             } else {
                 if (delta > 0.0) atomicAdd(&st->n_viol, 1ull);
                 copies = lnU < delta ? 1ull : 0ull;
@@ -1246,14 +1300,8 @@ __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t
         slot0 = __shfl_sync(0xffffffffu, slot0, 0);
         unsigned char *rec = nullptr;
         if (copies > 0) {
-            const float u0 = (float)((double)P->u0s * u0raw * inv), u2 = u0 * u0;
-            atomicAdd(&st->n_acc, copies);
-            atomicAdd(&st->hist[hist_bin(u0, __ldg(&P->hist_a), __ldg(&P->hist_b))], copies);
-            atomicAdd(&st->exc[exc_bin(u0, __ldg(&P->exc_a))], copies);
-            atomicAdd(&st->q[0], copies * (unsigned long long)__float2ll_rn(u0 * kQ1));
-            atomicAdd(&st->q[1], copies * (unsigned long long)__float2ll_rn(u2 * kQ2));
-            atomicAdd(&st->q[2], copies * (unsigned long long)__float2ll_rn(u2 * u0 * kQ3));
-            atomicAdd(&st->q[3], copies * (unsigned long long)__float2ll_rn(u2 * u2 * kQ4));
+            const float u0 = (float)((double)P->u0s * u0raw * inv);
+            tally_copies(st, P, u0, copies);
             const unsigned long long slot = slot0 + __popc(mk & ((1u << lane) - 1u));
             if (slot < B.ring_cap) {
                 rec = B.ring + slot * B.rec_bytes;
