@@ -244,10 +244,13 @@ struct GridRow {
 // (A second A tile per warpgroup, drawing tile t+1 before waiting for the
 // products of tile t, measured 8 % slower at three warpgroups than one tile
 // with the product-free decision terms made before the wait.)
-// HEADS: see k_sample_triad; here with three and four warpgroups (32 modes 12.93
-// -> 13.00e9 and 12.11 -> 12.19e9, 16 modes 21.1 -> 21.8e9 proposals/s; with two
-// warpgroups 10.71 -> 10.40e9, and 5.61 -> 5.08e9 at 64 modes).
-template <int KMAX, bool UNIF, int NWG, int UNR, bool HEADS = (NWG >= 3)>
+// The Philox blocks come from the chunk's table of heads (k_sample_triad's
+// HEADS; 32 modes 12.93 -> 13.00e9 and 12.11 -> 12.19e9, 16 modes 21.1 -> 21.8e9
+// proposals/s with four and three warpgroups).  With two warpgroups, two warps
+// per scheduler, a load in front of every block stands out (5.61 -> 5.08e9 at 64
+// modes), so there the heads of the next four blocks are loaded while four are
+// made (PF: 5.92e9).
+template <int KMAX, bool UNIF, int NWG, int UNR>
 __global__ void __launch_bounds__(128 * NWG, 1)
     k_sample_grid(const __grid_constant__ DevBufs B, const __grid_constant__ RunArgs A, uint32_t k0, uint32_t k1,
                   const unsigned char *__restrict__ bimg, int gridN) {
@@ -363,7 +366,7 @@ __global__ void __launch_bounds__(128 * NWG, 1)
             const float S = Sraw * inv2;
             const float tS = sc.cS * S;
             const float tQ = UNIF ? 0.f : sc.cQ * logf(zz * inv2);
-            const uint32_t wa = PhiloxOf<HEADS>(lo, hi, sc.pid, A.rk.k, W.heads).block((uint32_t)((sc.K + 1) / 2)).x;
+            const uint32_t wa = PhiloxTable(lo, hi, A.rk.k, W.heads).block((uint32_t)((sc.K + 1) / 2)).x;
             const float lnU = -0.5f * rho_fast(wa);
             // ---- 3. wait for the products, sum 2 C (C^2 + 3 S^2) of this row
             float cube = 0.f;
@@ -461,15 +464,12 @@ __global__ void __launch_bounds__(128 * NWG, 1)
                 nacc += (uint32_t)__popc(ma);
             }
         };
-        // with heads the chunk in one part, or in two where its indices cross a
-        // multiple of 2^32 (the heads hold for one upper half)
+        // the chunk in one part, or in two where its indices cross a multiple of
+        // 2^32 (the heads hold for one upper half)
         for (uint32_t i1 = 0, end = n_here; i1 < n_here; i1 = end) {
-        if constexpr (HEADS) {
-            end = i1 + (uint32_t)umin64(n_here - i1, 0x100000000ull - (uint32_t)(cbase + i1));
-            if (i1) wg_sync(g);  // the first part's readers of the heads are done
-            if (t <= KMAX / 2)
-                W.heads[t] = philox_head((uint32_t)t, (uint32_t)((cbase + i1) >> 32), sc.pid, A.rk.k);
-        }
+        end = i1 + (uint32_t)umin64(n_here - i1, 0x100000000ull - (uint32_t)(cbase + i1));
+        if (i1) wg_sync(g);  // the first part's readers of the heads are done
+        if (t <= KMAX / 2) W.heads[t] = philox_head((uint32_t)t, (uint32_t)((cbase + i1) >> 32), sc.pid, A.rk.k);
         wg_sync(g);
         const uint32_t n_tiles = (end - i1 + 127u) / 128u;
         for (uint32_t trip = 0; trip < n_tiles; ++trip) {
@@ -483,14 +483,34 @@ __global__ void __launch_bounds__(128 * NWG, 1)
                 // the mode sums over even and odd modes in packed pairs
                 f32x2_t nrm2p = 0ull, Srawp = 0ull, zzp = 0ull, esump = 0ull;
                 uint32_t wmin = 0xFFFFFFFFu;
-                const PhiloxOf<HEADS> prow(lo, hi, sc.pid, A.rk.k, W.heads);
+                const PhiloxTable prow(lo, hi, A.rk.k, W.heads);
+                constexpr bool PF = NWG < 3;
+                uint4 hn[4];
+                if constexpr (PF) {
+#pragma unroll
+                    for (int jj = 0; jj < 4; ++jj) hn[jj] = *reinterpret_cast<const uint4 *>(&W.heads[jj]);
+                }
 #pragma unroll(UNR)
                 for (int c8 = 0; c8 < KMAX / 8; ++c8) {
                     float vx[8], vy[8];
+                    uint4 hc[4];
+                    if constexpr (PF) {
+#pragma unroll
+                        for (int jj = 0; jj < 4; ++jj) hc[jj] = hn[jj];
+                        if (c8 + 1 < KMAX / 8) {
+#pragma unroll
+                            for (int jj = 0; jj < 4; ++jj)
+                                hn[jj] = *reinterpret_cast<const uint4 *>(&W.heads[4 * c8 + 4 + jj]);
+                        }
+                    }
 #pragma unroll
                     for (int jj = 0; jj < 4; ++jj) {
                         const int j = 4 * c8 + jj;
-                        const uint4 w = prow.block((uint32_t)j);
+                        uint4 w;
+                        if constexpr (PF)
+                            w = prow.tail.block(PhiloxHead{hc[jj].x, hc[jj].y, hc[jj].z, hc[jj].w});
+                        else
+                            w = prow.block((uint32_t)j);
                         const float4 c0 = W.mp[j][0], c1 = W.mp[j][1];
                         const f32x2_t s2 = pk2(c0.x, c0.y);
                         f32x2_t rho2, rr2, x2, y2;
