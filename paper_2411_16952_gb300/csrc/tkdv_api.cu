@@ -291,15 +291,40 @@ int build_args(tkdv_sampler *h, const unsigned long long *idx0, const unsigned l
         a.count[p] = count[p];
         total += count[p];
     }
-    // about 8 chunks per persistent worker (a CTA of the triad form, a
-    // warpgroup of the grid form), between 1 and 64 proposals per thread
-    const bool grid = is_grid(h);
+    // Chunks: a whole number m of them per persistent worker (a CTA of the
+    // triad form, a warpgroup of the grid form), between 1 and 64 proposals per
+    // thread, so that the last round is full: 8, or more where 64 proposals
+    // per thread are not enough; in the triad form, whose CTAs do not share an
+    // SM's issue slots as warpgroups do, 32 or 16 where a chunk still has 16
+    // trips of the CTA's loop.  With the largest chunks whatever the count,
+    // 2^25 proposals at 64 modes were 13.5 rounds that took 14 (6.22 -> 6.12
+    // ms), 8 x 2^22 in the triad form 6.7 that took 7 (3.43 -> 3.37 ms), 2 x
+    // 2^21 at 128 modes 7.7 that took 8 (3.41 -> 3.31 ms).
+    const bool grid = is_grid(h), warp = h->kmax == 128;
     const unsigned long long thr = grid ? 128ull : (unsigned long long)h->launch.threads;
+    const unsigned long long trip = warp ? 32ull : thr;  // (the warp form: four proposals per warp)
     const unsigned long long workers =
         (unsigned long long)h->launch.ctas * (grid ? (unsigned long long)h->kg.nwg[h->launch.variant] : 1ull);
-    unsigned long long target = (total + 8ull * workers - 1) / (8ull * workers);
-    target = (target + thr - 1) / thr * thr;
-    target = std::max(thr, std::min(thr * 64ull, target));
+    unsigned long long target;
+    if (h->opt.sir) {
+        // the FP32 partial sums of a chunk, and so the last bits of the
+        // importance sums, depend on its size: left as it was
+        target = (total + 8ull * workers - 1) / (8ull * workers);
+        target = (target + thr - 1) / thr * thr;
+        target = std::max(thr, std::min(thr * 64ull, target));
+    } else {
+        const unsigned long long per = (total + workers - 1) / workers, most = thr * 64ull;
+        unsigned long long m = 8;
+        if (!grid && !warp) m = per >= 32 * 16 * trip ? 32 : per >= 16 * 16 * trip ? 16 : 8;
+        m = std::max(m, (per + most - 1) / most);
+        // every point may end in a chunk that is not full
+        const unsigned long long chunks = workers * m, rest = (unsigned long long)h->n_points - 1;
+        target = (total + chunks - 1) / chunks;
+        if (chunks > 2 * rest) target = (total + (chunks - rest) - 1) / (chunks - rest);
+        target = (target + trip - 1) / trip * trip;
+        target = std::max(warp ? trip : thr, std::min(most, target));
+        if (m > 1024) target = most;  // the round does not matter, the chunk count might
+    }
     a.chunk = (uint32_t)target;
     unsigned long long acc = 0;
     a.chunk_prefix[0] = 0;
