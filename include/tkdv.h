@@ -191,8 +191,8 @@ typedef struct tkdv_sampler tkdv_sampler;
 
 /* sampler_create: one parameter point with default options (K given here,
    triad H3, 2^20-record ring, own stream).  Runs the per-point precompute of
-   Sec. IV.B on the host: alpha* (Eq. 29), sigma_k (Eq. 25) and log M
-   (Eq. 45), then allocates device buffers.  The 4th argument is C3/C2.
+   Sec. IV.B: alpha* (Eq. 29) and sigma_k (Eq. 25) on the host, log M (Eq. 45)
+   on the device once its buffers are allocated.  The 4th argument is C3/C2.
    Errors: INVALID_ARG (K outside 1..128, E0 <= 0, beta' < 0, unknown
    proposal), NO_ALPHA, OOM, CUDA.  *out is NULL on error. */
 int sampler_create(int K, double beta_p, double E0, double r, int proposal, tkdv_sampler **out);

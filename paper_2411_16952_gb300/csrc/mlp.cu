@@ -691,6 +691,7 @@ int tkdv_mlp_rows(tkdv_mlp *m, uint64_t *counts) {
 
 int tkdv_mlp_step(tkdv_mlp *m, float lr, float tau, int update, double *loss, float *grad_out) {
     if (!m || m->P < 1) return TKDV_ERR_INVALID_ARG;
+    if (!m->d_done) return mfail(m, TKDV_ERR_INVALID_ARG, "the training set was refused");  // (allocated last)
     const int P = m->P;
     const __nv_bfloat16 *wb = m->d_wb[m->cur];
     k_forward<<<P, 64>>>(wb, m->d_feats, m->d_h1, m->d_h2, m->d_out, m->d_K, m->d_wpaper, m->d_wprime, m->d_slw);

@@ -75,10 +75,10 @@ void fill_point_const(int K, const tkdv_point &q, const double *s2, double logM,
     //
     // The warp form (K > 64, sampler_k128.cu) sums differently: a mode sum
     // (|x|^2, S|x|^2, Q|x|^2) passes each term through at most 12 roundings
-    // (its own 3, 4 per lane, 5 in the warp tree), a triad term through at most
-    // 50 (8 on its anti-diagonal, 31 in its tile, 3 over rounds, 5 in the warp
-    // tree, 3 in the scaling), so chains of 32 and 64 replace 2K + 16; the
-    // hardware sine and cosine add at most 2^-21.4 = 6.1 ulp per component,
+    // (its own 3, 4 per lane, 5 in the warp tree); T, by the transform of
+    // sampler_k128.cu, moves by at most 75 eps sqrt(K) through its roundings.
+    // Chains of 32 and 64 (512 eps sqrt(K) with the factor eight) replace
+    // 2K + 16; the hardware sine and cosine add at most 2^-21.4 = 6.1 ulp per component,
     // well inside the factor eight.  Its radius -2 logf(u) has no absolute
     // error and a relative one below kRhoLogRelErr, so the per-draw terms (3)
     // vanish.
