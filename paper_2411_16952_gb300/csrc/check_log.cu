@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(256) k_check_rho(unsigned long long *worst) {
     const uint32_t w = m << 9;  // any word of bucket m
     const double u = (2.0 * (double)m + 1.0) * 0x1p-24;
     const double ref = -2.0 * log(u);
-    // rho_fast is rho_raw or its floor: the larger of their errors
+    // (one-thread form: the larger of the errors of rho_raw and rho_fast)
     const double got = LOG ? (double)rho_log(w) : (double)rho_raw(w);
     const double bound = LOG ? kRhoLogRelErr * ref : kRhoAbsErr + kRhoRelErr * ref;
     double err = got > 0.0 ? fabs(got - ref) / bound : INFINITY;  // (its square root is taken)
