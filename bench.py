@@ -48,26 +48,32 @@ def measured_peaks():
 def alg_ops_per_proposal(K: int, form: str = "triad", grid_N: int = 128) -> int:
     """Ideal thread-instruction count of one proposal.
 
-    Both forms: Philox4x32-10 (ceil(K/2)+1 blocks x 10 rounds x 4: two wide
-    multiplies and two 3-input xors) and 40 for log Q, ln U, the ratio and
-    the decision.
+    All forms: Philox4x32-10, ceil(K/2)+1 blocks of 33 (15 wide multiplies and
+    17 3-input xors with the first rounds shared by a run, one load of the
+    shared words) and 40 for log Q, ln U, the ratio and the decision.
     triad (scalar FP32 per mode): Box-Muller and sigma scaling (20 per mode),
     the |x|^2, S, Q, u0 accumulations (4 per mode), and the symmetric double
     sum of Eq. (42) in packed FP32x2 pairs (2 per pair k < n-k, 4 for the
     middle term of an even n and 2 for the doubling of an odd one, 4 for the
-    outer update); the same count serves the warp form (K > 64).
+    outer update).
+    warp (K > 64): the same draw, and H3 by the transform onto 384 points: 24
+    columns of 115 (11 coefficient sums, 22 for the twists by constants, 50
+    for eight points, 32 for the twists) and 8 rows of 348 (eight 3-point
+    transforms of 12, three 8-point ones of 52, 24 cubes of 4).
     grid (the two modes of a Philox block in packed FP32x2 pairs where the
-    data allow): per pair of modes 22 for Box-Muller and scaling (4 bit
-    shifts, 2 lg2, 2 floors, 2 rsqrt, 4 sin/cos, 8 packed multiply/add),
-    4 packed accumulations, 2 table loads and 2 minima of the radius words;
-    per value 2.5 for the BF16 hi/lo split (packed residuals) and 0.25 for
-    the 16-byte shared-memory stores; 1.5 per mirror pair of grid points
-    for 2 C (C^2 + S'^2) (three packed instructions per two pairs); one
-    TMEM load per 16 columns of C and of S.  20.5 per mode in all."""
+    data allow): per pair of modes 20 for Box-Muller and scaling (4 bit
+    shifts, 2 lg2, 2 rsqrt, 4 sin/cos, 8 packed multiply/add), 4 packed
+    accumulations, 2 table loads and 2 minima of the radius words; per value
+    2.5 for the BF16 hi/lo split (packed residuals) and 0.25 for the 16-byte
+    shared-memory stores; 1.5 per mirror pair of grid points for
+    2 C (C^2 + S'^2) (three packed instructions per two pairs); one TMEM load
+    per 16 columns of C and of S.  19.5 per mode in all."""
     blocks = (K + 1) // 2 + 1
     if form == "grid":
-        return int(40 * blocks + 20.5 * K + 0.75 * grid_N + grid_N // 16 + 40)
-    common = 40 * blocks + 20 * K + 4 * K + 40
+        return int(33 * blocks + 19.5 * K + 0.75 * grid_N + grid_N // 16 + 40)
+    common = 33 * blocks + 20 * K + 4 * K + 40
+    if form == "warp":
+        return common + 24 * 115 + 8 * 348
     triad = sum(2 * ((n - 1) // 2) + (4 if n % 2 == 0 else 2) + 4 for n in range(2, K + 1))
     return common + triad
 
@@ -78,13 +84,13 @@ def alg_ops_per_proposal(K: int, form: str = "triad", grid_N: int = 128) -> int:
 # read no per-proposal input, so traffic scales with the proposals processed.
 # Set to None whenever the kernel changes until it is captured again.
 TRAFFIC_PER_PROPOSAL = {
-    "grid": (137984.0 / (8 * 4194304),
+    "grid": (140032.0 / (8 * 4194304),
              "ncu --set full capture prof_grid_k32 (k_sample_grid<32,0,4,4>, 8 x 2^22 proposals)"),
-    "triad": (116736.0 / (8 * 4194304),
-              "ncu --set full capture prof_triad (k_sample_triad<32,0,256,1,0,1>, 8 x 2^22 proposals)"),
+    "triad": (118784.0 / (8 * 4194304),
+              "ncu --set full capture prof_triad (k_sample_triad<32,0,256,2,0,1,1>, 8 x 2^22 proposals)"),
 }
 # the 64-mode grid kernel: one capture of the upstream run at 2^26 proposals
-TRAFFIC_PER_PROPOSAL_K64 = (184576.0 / (1 << 26),
+TRAFFIC_PER_PROPOSAL_K64 = (175616.0 / (1 << 26),
                             "ncu --set full capture prof_grid_k64 (k_sample_grid<64,0,2,2>, 2^26 proposals)")
 
 
@@ -696,7 +702,7 @@ def main():
         kst = SK.stats()
         kprop = sum(s["n_proposals"] for s in kst)
         kacc = sum(s["n_accepted"] for s in kst)
-        kops = alg_ops_per_proposal(kw["K"], "triad")
+        kops = alg_ops_per_proposal(kw["K"], "warp")
         kpeak = alu_peak(n_sms, peaks)
         kpps = kprop / (kms * args.steps / 1e3)
         k128 = {"workload": kw["name"], "K": kw["K"], "ms_per_step": kms, "proposals_per_s": kpps,
