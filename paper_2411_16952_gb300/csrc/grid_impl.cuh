@@ -249,7 +249,7 @@ struct GridRow {
 // proposals/s with four and three warpgroups).  With two warpgroups, two warps
 // per scheduler, a load in front of every block stands out (5.61 -> 5.08e9 at 64
 // modes), so there the heads of the next four blocks are loaded while four are
-// made (PF: 5.92e9).
+// made (PF: 5.92e9; 5.84e9 since the radius has its offset).
 template <int KMAX, bool UNIF, int NWG, int UNR>
 __global__ void __launch_bounds__(128 * NWG, 1)
     k_sample_grid(const __grid_constant__ DevBufs B, const __grid_constant__ RunArgs A, uint32_t k0, uint32_t k1,
