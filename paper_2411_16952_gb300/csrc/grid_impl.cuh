@@ -312,8 +312,7 @@ __global__ void __launch_bounds__(128 * NWG, 1)
     const uint32_t mbar = smem_u32(&s_mbar[g]);
     uint32_t phase = 0;
     bool pending = false;  // an MMA commit of this warpgroup not yet waited for
-    // this warp's slab: room for the accepted draws of one chunk (at most
-    // chunk / 4 proposals per warp)
+    // this warp's slab: room for the accepted draws of one chunk (kAcceptSlab)
     AcceptItem *slab = B.accs + ((size_t)(blockIdx.x * NWG + g) * 4 + (size_t)(t >> 5)) * B.acc_slab;
     const float tscale = 8.f / (3.f * (float)gridN);  // T = (4/(3N)) sum U^3/|x|^3, sum U^3 = 2 sum C (C^2 + 3 S^2)
 

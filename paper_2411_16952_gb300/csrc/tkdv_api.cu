@@ -311,9 +311,9 @@ int build_args(tkdv_sampler *h, const unsigned long long *idx0, const unsigned l
         // importance sums, depend on its size: left as it was
         target = (total + 8ull * workers - 1) / (8ull * workers);
         target = (target + thr - 1) / thr * thr;
-        target = std::max(thr, std::min(thr * 64ull, target));
+        target = std::max(thr, std::min(thr * kChunkPerThread, target));
     } else {
-        const unsigned long long per = (total + workers - 1) / workers, most = thr * 64ull;
+        const unsigned long long per = (total + workers - 1) / workers, most = thr * kChunkPerThread;
         unsigned long long m = 8;
         if (!grid && !warp) m = per >= 32 * 16 * trip ? 32 : per >= 16 * 16 * trip ? 16 : 8;
         m = std::max(m, (per + most - 1) / most);

@@ -16,9 +16,13 @@ constexpr int kMaxPoints = 64;
 constexpr int kHistBins = 256;
 constexpr int kExcBins = 26;  // exceed-bin e = number of thresholds 0.25 i sigma0 below u0
 constexpr uint32_t kRefineCap = 1u << 22;
-// grid form: accepted draws one warp holds until the end of its chunk (a
-// chunk has at most 64 proposals per thread, so 2048 per warp)
-constexpr uint32_t kAcceptSlab = 2048;
+// Most proposals per thread in one chunk.
+constexpr uint32_t kChunkPerThread = 64;
+// grid form: accepted draws one warp holds until the end of its chunk, 32 of
+// each tile of 128 proposals.  A chunk whose indices cross a multiple of 2^32
+// is taken in two parts that each end in a tile of their own, so a full chunk
+// can have one tile more than its proposals per thread.
+constexpr uint32_t kAcceptSlab = 32 * (kChunkPerThread + 1);
 
 // Fixed-point scales of the u0^p moment sums (exact 64-bit integer sums).
 constexpr float kQ1 = 268435456.0f;  // 2^28
