@@ -200,6 +200,7 @@ int set_form(tkdv_sampler *h, int form) {
     h->pc = form == TKDV_H3_GRID_BF16X3 ? h->pc_grid : h->pc_triad;
     CK(cudaStreamSynchronize(h->stream));
     CK(cudaMemcpy(h->d_pts, h->pc.data(), sizeof(PointConst) * h->n_points, cudaMemcpyHostToDevice));
+    CK(cudaStreamSynchronize(cudaStreamLegacy));  // (the copy may return before it has run)
     if (form == TKDV_H3_GRID_BF16X3) {
         h->launch.variant = h->gfirst;
         h->launch.threads = variant_threads(h, h->gfirst);
@@ -451,7 +452,7 @@ struct StateTail {
 size_t state_bytes(const tkdv_sampler *h) { return sizeof(StatBlock) * (size_t)h->n_points + sizeof(StateTail); }
 
 int check_status(tkdv_sampler *h, uint32_t st) {
-    if (st) CK(cudaMemset(h->d_status, 0, 4));
+    if (st) CK(cudaMemsetAsync(h->d_status, 0, 4, h->stream));
     if (st & (kStatusDeadline | kStatusMbarTimeout))
         return fail(h, TKDV_ERR_TIMEOUT,
                     (st & kStatusDeadline) ? "run stopped at its deadline" : "device wait timed out");
@@ -699,6 +700,9 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
     h->pc = h->launch.form == TKDV_H3_GRID_BF16X3 ? h->pc_grid : h->pc_triad;
     e = cudaMemcpy(h->d_pts, h->pc.data(), sizeof(PointConst) * n_points, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(h->d_stats, 0, state_bytes(h));
+    // nothing orders the legacy stream's copies and memsets, which may return
+    // before they have run, with the runs on the handle's stream
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         h->err = std::string("initialising device buffers: ") + cudaGetErrorString(e);
         return bail(TKDV_ERR_CUDA);
@@ -942,7 +946,9 @@ int sampler_extreme_field(tkdv_sampler *h, int point, uint64_t m, uint64_t max_r
 int sampler_reset(tkdv_sampler *h) {
     if (!h) return TKDV_ERR_INVALID_ARG;
     CK(cudaStreamSynchronize(h->stream));
-    CK(cudaMemset(h->d_stats, 0, state_bytes(h)));
+    // on the stream of the runs: one of the legacy stream would wait behind
+    // other work there and clear the state of a run that has begun
+    CK(cudaMemsetAsync(h->d_stats, 0, state_bytes(h), h->stream));
     std::fill(h->next_idx.begin(), h->next_idx.end(), 0ull);
     return TKDV_OK;
 }
