@@ -857,6 +857,16 @@ int sampler_samples(tkdv_sampler *h, void *dst, int dst_on_device, uint64_t max_
     n = std::min<unsigned long long>(n, max_records);
     if (n) CK(cudaMemcpy(dst, h->d_ring, n * h->rec_bytes, dst_on_device ? cudaMemcpyDeviceToDevice
                                                                            : cudaMemcpyDeviceToHost));
+    if (n && dst_on_device) {
+        // a copy on the device does not hold the host: the next run on the
+        // handle's stream waits before it writes the ring
+        cudaEvent_t copied;
+        CK(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming));
+        cudaError_t e = cudaEventRecord(copied, cudaStreamLegacy);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, copied, 0);
+        cudaEventDestroy(copied);
+        CK(e);
+    }
     *n_out = n;
     return TKDV_OK;
 }

@@ -66,3 +66,25 @@ def test_a_new_handle_is_initialised_before_its_first_run(env, form):
         ref = ref or got
         for a, b in zip(ref, got):
             assert np.array_equal(a, b)
+
+
+def test_records_copied_on_the_device_are_those_of_the_finished_run(env):
+    torch, T = env
+    # every proposal is accepted (beta' = 0, uniform): both runs fill the ring
+    cap, K = 1 << 20, 64
+    S = T.Sampler(K, [T.make_point(0.0, 1.0, 0.0, T.PROPOSAL_UNIFORM, logM=0.0)], sample_capacity=cap)
+    buf = torch.zeros(cap * T.tkdv_record_bytes(K), dtype=torch.uint8, device="cuda")
+    want = torch.zeros_like(buf)
+    for seed in (1, 2, 3):
+        S.reset()
+        S.run(cap, seed)
+        S.sync()
+        assert S.samples(cap, device_dst=want) == cap
+        torch.cuda.synchronize()
+        assert S.samples(cap, device_dst=buf) == cap
+        S.reset()
+        S.run(cap, seed + 100)  # while the copy of 570 MB is on its way
+        S.sync()
+        torch.cuda.synchronize()
+        assert torch.equal(buf, want)
+    S.close()
