@@ -605,6 +605,9 @@ class Sampler:
         of `point` (by proposal index) the one with the largest displacement
         on the 2K-point grid.  Returns a dict (idx, umax, xi, xhat) or None
         when fewer than m fields were kept."""
+        # as numbers compare: C would cut point 2^32 to 0, m = 2^64 + 1 to 1
+        point = next((p for p in range(self.n_points) if p == point), -1)
+        m = min(m, 1 << 62)
         if m < 0:  # all but the last -m
             m = max(0, sampler_extreme_field(self.h, self.K, point, 1 << 62, max_records)[0] + m)
         if m == 0:
