@@ -251,8 +251,10 @@ int sampler_field_maxima(tkdv_sampler *h, uint64_t max_records, double *umax, in
    floats, [cosine | sine]) describe it; all are host pointers.  *n_found
    receives the number of fields of the point among those records; when it is
    below m (m >= 1) nothing else is written.  Runs on the handle's stream
-   (synchronises) in the handle's buffers; allocates device memory for the
-   call only above 4M records.  Errors: INVALID_ARG, OOM, CUDA. */
+   (synchronises) in 64 MB of the handle's buffers; allocates device memory
+   for the call where the selection needs more: 16 bytes per record of the
+   first min(max_records, kept), 24 per field of the m (none where m is above
+   the number of records) and 9 KB.  Errors: INVALID_ARG, OOM, CUDA. */
 int sampler_extreme_field(tkdv_sampler *h, int point, uint64_t m, uint64_t max_records, uint64_t *idx, double *umax,
                           int32_t *jmax, float *xhat, uint64_t *n_found);
 

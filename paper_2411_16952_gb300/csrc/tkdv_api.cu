@@ -914,8 +914,9 @@ int sampler_extreme_field(tkdv_sampler *h, int point, uint64_t m, uint64_t max_r
     n = std::min<unsigned long long>(n, max_records);
     *n_found = 0;
     if (!n || point < 0 || point >= h->n_points) return TKDV_OK;
-    // the FP64 queue is free between runs; a larger ring gets its own scratch
-    const unsigned long long mm = std::min<unsigned long long>(m, n);
+    // more fields than records are never found: only the count is wanted then.
+    // The FP64 queue is free between runs; what it cannot hold gets its own scratch.
+    const unsigned long long mm = m > n ? 1 : m;
     const size_t need = extreme_scratch_bytes(n, mm);
     void *scratch = h->d_refine, *own = nullptr;
     if (need > sizeof(RefineItem) * (size_t)kRefineCap) {
