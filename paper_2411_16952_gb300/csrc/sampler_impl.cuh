@@ -1110,12 +1110,12 @@ __device__ __forceinline__ void tally_copies(StatBlock *st, const PointConst *P,
 }
 
 // ---- FP64 decision of the guard-band proposals ---------------------------
-// A CTA takes up to 32 queued proposals.  The K modes of a proposal and its
-// triads are spread over a segment of kLanes lanes of a warp (32 / kLanes
-// proposals at a time, the four warps in turn), and their sums meet in the
-// segment by shuffles; the scalar part of the decision (1/|x|, the logarithms,
-// the SIR copy number) then runs once for the whole batch, a proposal per lane
-// of the first warp.
+// A group of four warps takes up to 32 queued proposals.  The K modes of a
+// proposal and its triads are spread over a segment of kLanes lanes of a warp
+// (32 / kLanes proposals at a time, the four warps in turn), and their sums meet
+// in the segment by shuffles; the scalar part of the decision (1/|x|, the
+// logarithms, the SIR copy number) then runs once for the whole batch, a
+// proposal per lane of one of the warps.
 //
 // What bounds it: an FP64 instruction of a warp holds its scheduler for 64
 // cycles (measured, dependent or not, whatever the number of active lanes).
@@ -1125,16 +1125,35 @@ __device__ __forceinline__ void tally_copies(StatBlock *st, const PointConst *P,
 // same FP64 work is about 400, 400 and 700 warp instructions: a run of 2^16
 // proposals at 16 modes went from 166 to 94 us (static call), one of 2^25 at
 // 64 modes from 7.04 to 6.40 ms, of 8 x 2^22 at 32 modes from 4.03 to 3.82 ms.
-// With a full queue both forms need about the same number of FP64 warp
-// instructions per proposal, so there is one form only.
+// Four groups share an SM's CTA, the decisions of each on another scheduler:
+// with one group the decisions left three schedulers idle, and 200,000 queued
+// proposals at 16 modes took 1,234 us, in an SIR run 3,970 (now 857 and 1,630).
+//
+// In a full queue every lane can have a proposal of its own, and where a segment
+// has lanes without a mode that takes less: one thread per proposal
+// (refine_serial) from 16 queued proposals a warp on, up to kSerialModes modes.
+// SIR runs that queue and keep 166,000 fields, us a run, batches against one per
+// thread: of eight points 1,133 and 854 at 4 modes, 1,146 and 1,026 at 8, 1,507
+// and 1,094 at 9, 1,564 and 1,392 at 14, 1,547 and 1,526 at 16, 2,111 and 1,600
+// at 17, 2,277 and 1,846 at 20, 2,266 and 2,173 at 24, 2,378 and 2,515 at 28, 2,437
+// and 2,898 at 32, 3,533 and 3,201 at 33, 3,566 and 3,437 at 36, 3,691 and 4,004 at
+// 40, 4,929 and 7,170 at 64; of one point, whose statistics all threads add to,
+// 1,143 and 1,066 at 4, 1,503 and 1,473 at 9, 1,545 and 2,070 at 14, 2,244 and 2,932
+// at 20, 2,274 and 3,579 at 24, 3,526 and 4,459 at 33, 4,962 and 9,730 at 64.  With
+// 20,000 queued by eight points 315 and 208 at 9, 412 and 271 at 17, 463 and 444 at
+// 32, 839 and 1,028 at 64; alone in the queue a proposal takes 14 and 84 at 16 modes.
 template <int KMAX>
 struct RefineShape {
     static constexpr int kLanes = KMAX < 8 ? 8 : KMAX < 32 ? KMAX : 32;  // lanes of one proposal
     static constexpr int kGroup = 32 / kLanes;                          // proposals at a time
     static constexpr int kModes = KMAX / kLanes > 1 ? KMAX / kLanes : 1;  // modes of one lane
     static constexpr int kBatch = 32;
-    static constexpr int kWarps = 4;
-    static constexpr size_t kSmem = sizeof(double2) * kBatch * KMAX;
+    static constexpr int kWarps = 4;   // warps of a batch, one per scheduler
+    static constexpr int kGroups = 4;  // batches of a CTA at a time
+    static constexpr int kThreads = 32 * kWarps * kGroups;
+    static constexpr size_t kSmem = sizeof(double2) * kBatch * KMAX * kGroups;
+    // the modes up to which a full queue is taken by one thread per proposal
+    static constexpr int kSerialModes = KMAX <= 8 ? KMAX : KMAX == 16 ? 14 : KMAX == 32 ? 20 : 34;
 };
 
 // Sums over a segment's lanes, the same values in every lane of it.
@@ -1145,13 +1164,15 @@ __device__ __forceinline__ double seg_sum(double v) {
     return v;
 }
 
-// The FP64 pass of an SIR run that queues more draws than the ring has room
-// for, one proposal per thread.  The records that do not fit are counted per
-// point, and which points they fall on follows the order in which draws
-// finish: consecutive draws together, as in this form.
+// One proposal per thread: full queues (RefineShape), and SIR runs that queue
+// more draws than the ring has room for.  The records that do not fit are
+// counted per point, and which points they fall on follows the order in which
+// draws finish: consecutive draws together, as in this form.
 template <int KMAX, bool UNIF>
 __device__ __noinline__ void refine_serial(const DevBufs &B, uint32_t n, uint32_t k0, uint32_t k1) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    // a short queue goes to the first warps of all CTAs, not to all warps of the first
+    for (uint32_t i = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31); i < n;
+         i += gridDim.x * blockDim.x) {
         const RefineItem it = B.refine[i];
         const PointConst *P = B.pts + it.point;
         StatBlock *st = B.stats + it.point;
@@ -1160,11 +1181,13 @@ __device__ __noinline__ void refine_serial(const DevBufs &B, uint32_t n, uint32_
         eval64<KMAX, UNIF>(P, it.idx, k0, k1, &o, xh);
         atomicAdd(&st->n_refined, 1ull);
         atomicMax(&st->maxd_key, (unsigned long long)fkey((float)o.delta));
-        bool near = false;
-        const unsigned long long copies = (unsigned long long)sir_copies(P->sir_c * exp(o.delta), o.u, o.lnU, near);
+        bool near = o.near;
+        unsigned long long copies = o.accept ? 1ull : 0ull;
+        if (B.sir) copies = (unsigned long long)sir_copies(P->sir_c * exp(o.delta), o.u, o.lnU, near);
         if (near) atomicAdd(&st->n_near, 1ull);
+        if (!B.sir && o.delta > 0.0) atomicAdd(&st->n_viol, 1ull);
         if (copies == 0) continue;
-        atomicAdd(&st->n_kept, 1ull);
+        if (B.sir) atomicAdd(&st->n_kept, 1ull);
         tally_copies(st, P, o.u0, copies);
         const int K = P->K;
         for (int m = 0; m < K; ++m)
@@ -1173,7 +1196,7 @@ __device__ __noinline__ void refine_serial(const DevBufs &B, uint32_t n, uint32_
         const unsigned long long slot = atomicAdd(B.ring_count, 1ull);
         if (slot < B.ring_cap) {
             unsigned char *rec = B.ring + slot * B.rec_bytes;
-            write_header(rec, it.idx, it.point, 1u | (near ? 2u : 0u) | (uint32_t)copies << 8, o.H2, o.H3, o.u0,
+            write_header(rec, it.idx, it.point, 1u | (near ? 2u : 0u) | (B.sir ? (uint32_t)copies << 8 : 0u), o.H2, o.H3, o.u0,
                          (float)o.delta);
             float *f = reinterpret_cast<float *>(rec + 32);
             for (int m = 0; m < 2 * K; ++m) f[m] = xh[m];
@@ -1184,24 +1207,26 @@ __device__ __noinline__ void refine_serial(const DevBufs &B, uint32_t n, uint32_
 }
 
 template <int KMAX, bool UNIF>
-__global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t k1) {
+__global__ void __launch_bounds__(RefineShape<KMAX>::kThreads) k_refine(DevBufs B, uint32_t k0, uint32_t k1) {
     using RS = RefineShape<KMAX>;
     constexpr int LANES = RS::kLanes, GROUP = RS::kGroup, MODES = RS::kModes;
     extern __shared__ __align__(16) unsigned char s_refine[];
-    __shared__ double s_sum[RS::kBatch][5];  // |x|^2, S|x|^2, Q|x|^2, u(0)|x|/u0s, T|x|^3
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double s_sums[RS::kGroups][RS::kBatch][5];  // |x|^2, S|x|^2, Q|x|^2, u(0)|x|/u0s, T|x|^3
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % RS::kWarps, grp = (threadIdx.x >> 5) / RS::kWarps;
     const int sub = lane / LANES, l = lane % LANES;
-    double2 *slab = reinterpret_cast<double2 *>(s_refine);
+    double2 *slab = reinterpret_cast<double2 *>(s_refine) + (size_t)grp * RS::kBatch * KMAX;
+    double(*s_sum)[5] = s_sums[grp];
+    auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(32 * RS::kWarps) : "memory"); };
     const uint32_t n = min(*(volatile uint32_t *)&B.counters[1], B.refine_cap);
-    if (B.sir && n > B.ring_cap) {
+    if ((n > gridDim.x * (RS::kThreads / 2) && B.pts->K <= RS::kSerialModes) || (B.sir && n > B.ring_cap)) {
         refine_serial<KMAX, UNIF>(B, n, k0, k1);
         return;
     }
-    // batches of consecutive items, as small as the CTAs allow
-    const uint32_t batch = min((n + gridDim.x - 1) / gridDim.x, (uint32_t)RS::kBatch);
-    for (uint32_t first = blockIdx.x * batch; first < n; first += gridDim.x * batch) {
+    // batches of consecutive items, as small as the groups allow
+    const uint32_t units = gridDim.x * RS::kGroups, batch = min((n + units - 1) / units, (uint32_t)RS::kBatch);
+    for (uint32_t first = ((uint32_t)grp * gridDim.x + blockIdx.x) * batch; first < n; first += units * batch) {
         const uint32_t cnt = min(batch, n - first);
-        __syncthreads();  // the slab's readers of the previous batch are done
+        group_sync();  // the slab's readers of the previous batch are done
 #pragma unroll 1
         for (uint32_t g0 = (uint32_t)warp * GROUP; g0 < cnt; g0 += RS::kWarps * GROUP) {
             const uint32_t q = min(g0 + (uint32_t)sub, cnt - 1);  // (an idle segment repeats the last item)
@@ -1236,16 +1261,25 @@ __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t
                 if (m < KMAX) sx[m] = v;
             }
             __syncwarp();
-            // T = sum over k <= l, k + l <= KMAX of w Re(v_k v_l conj(v_{k+l})),
-            // w = 2 for k < l, else 1.  Row k holds the KMAX - 2k + 1 values
-            // l = k..KMAX-k; rows k and KMAX/2 + 1 - k together hold KMAX, so
-            // the KMAX^2/4 triads are numbered by (row pair, place in it).
+            // T = sum over k <= l, k + l <= N of w Re(v_k v_l conj(v_{k+l})),
+            // w = 2 for k < l, else 1, N = K or K + 1, the even one (mode K + 1
+            // is zero).  Row k holds the N - 2k + 1 values l = k..N-k; rows k
+            // and N/2 + 1 - k together hold N, so the N^2/4 triads are numbered
+            // by (row pair rp, place c in it).  (With N = KMAX whatever K the
+            // pass took half as long again at 33 modes.)
             double at = 0.0;
+            const int N = (K + 1) & ~1;
+            int rp = 0, c = l;
 #pragma unroll 2
-            for (int e = l; e < KMAX * KMAX / 4; e += LANES) {
-                const int rp = e / KMAX, c = e % KMAX, len = KMAX - 2 * rp - 1;
-                const int kk = c < len ? rp + 1 : KMAX / 2 - rp;
+            for (int e = l; e < N * N / 4; e += LANES) {
+                while (c >= N) {
+                    c -= N;
+                    ++rp;
+                }
+                const int len = N - 2 * rp - 1;
+                const int kk = c < len ? rp + 1 : N / 2 - rp;
                 const int ll = c < len ? kk + c : kk + (c - len);
+                c += LANES;
                 const double2 a = sx[kk - 1], b = sx[ll - 1], v = sx[kk + ll - 1];
                 const double A = fma(a.x, b.x, -(a.y * b.y)), Bv = fma(a.x, b.y, a.y * b.x);
                 at = fma(kk < ll ? 2.0 : 1.0, fma(v.x, A, v.y * Bv), at);
@@ -1264,8 +1298,8 @@ __global__ void __launch_bounds__(128) k_refine(DevBufs B, uint32_t k0, uint32_t
                 d[4] = at;
             }
         }
-        __syncthreads();
-        if (warp > 0) continue;
+        group_sync();
+        if (warp != grp % RS::kWarps) continue;  // (another scheduler for each group's decisions)
         // the decision of item first + lane (the formulas of eval64)
         const bool valid = (uint32_t)lane < cnt;
         const double *sums = s_sum[min((uint32_t)lane, cnt - 1)];
@@ -1430,6 +1464,8 @@ void fill_triad_kernels_xfer(TriadKernels *t) {
     t->refine[0] = (const void *)k_refine<KMAX, false>;
     t->refine[1] = (const void *)k_refine<KMAX, true>;
     t->refine_smem = (int)RefineShape<KMAX>::kSmem;
+    t->refine_threads = RefineShape<KMAX>::kThreads;
+    t->refine_ctas = 1;
     t->replay[0] = (const void *)k_replay<KMAX, false>;
     t->replay[1] = (const void *)k_replay<KMAX, true>;
     t->replay_per_block = 128;

@@ -806,6 +806,8 @@ void triad_kernels_k128(TriadKernels *t) {
     t->refine[0] = (const void *)k_refine_warp<false>;
     t->refine[1] = (const void *)k_refine_warp<true>;
     t->refine_smem = 0;
+    t->refine_threads = 128;
+    t->refine_ctas = 4;
     t->replay[0] = (const void *)k_replay_warp<false>;
     t->replay[1] = (const void *)k_replay_warp<true>;
     t->replay_per_block = 32 * kReplayWarps / 32 * kWQ;

@@ -343,10 +343,8 @@ int build_args(tkdv_sampler *h, const unsigned long long *idx0, const unsigned l
     return TKDV_OK;
 }
 
-// CTAs of the FP64 pass.  The one-thread forms' k_refine fills the FP64 pipes
-// with one warp per scheduler, so one CTA of four warps per SM; the warp form's
-// k_refine_warp takes one proposal per warp and four CTAs per SM.
-int refine_grid(tkdv_sampler *h) { return std::max(1, h->num_sms * (h->kt.refine_smem ? 1 : 4)); }
+// CTAs of the FP64 pass (k_refine, k_refine_warp).
+int refine_grid(tkdv_sampler *h) { return std::max(1, h->num_sms * h->kt.refine_ctas); }
 
 int build_graph(tkdv_sampler *h) {
     if (h->exec) {
@@ -382,7 +380,7 @@ int build_graph(tkdv_sampler *h) {
     cudaKernelNodeParams rp{};
     rp.func = (void *)h->kt.refine[uni];
     rp.gridDim = dim3(refine_grid(h));
-    rp.blockDim = dim3(128);
+    rp.blockDim = dim3(h->kt.refine_threads);
     rp.sharedMemBytes = (unsigned)h->kt.refine_smem;
     rp.kernelParams = rargs;
     CK(cudaGraphAddKernelNode(&h->n_refine, h->graph, &h->n_main, 1, &rp));
@@ -413,7 +411,7 @@ int enqueue(tkdv_sampler *h) {
         cudaKernelNodeParams rp{};
         rp.func = (void *)h->kt.refine[uni];
         rp.gridDim = dim3(refine_grid(h));
-        rp.blockDim = dim3(128);
+        rp.blockDim = dim3(h->kt.refine_threads);
         rp.sharedMemBytes = (unsigned)h->kt.refine_smem;
         rp.kernelParams = rargs;
         CK(cudaGraphExecKernelNodeSetParams(h->exec, h->n_refine, &rp));
@@ -427,7 +425,7 @@ int enqueue(tkdv_sampler *h) {
     CK(cudaLaunchKernel(main_fn(h, h->launch.variant), dim3(h->launch.ctas), dim3(h->launch.threads), margs,
                         main_dyn_smem(h, h->launch.variant, h->launch.threads), h->stream));
     void *rargs[] = {&h->dev, &h->key0, &h->key1};
-    CK(cudaLaunchKernel(h->kt.refine[uni], dim3(refine_grid(h)), dim3(128), rargs, (size_t)h->kt.refine_smem, h->stream));
+    CK(cudaLaunchKernel(h->kt.refine[uni], dim3(refine_grid(h)), dim3(h->kt.refine_threads), rargs, (size_t)h->kt.refine_smem, h->stream));
     return TKDV_OK;
 }
 

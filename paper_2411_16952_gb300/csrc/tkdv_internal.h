@@ -154,7 +154,7 @@ struct TriadKernels {
     int n_variants;  // variants present (6, or 3 for the warp form)
     const void *sir[2];  // SIR form of the sampler (256 threads), [uniform]
     const void *refine[2];
-    int refine_smem;  // dynamic shared memory of one refine CTA (128 threads)
+    int refine_smem, refine_threads, refine_ctas;  // dynamic shared memory and threads of a refine CTA, CTAs per SM
     const void *replay[2];
     int replay_per_block;  // indices one replay CTA of 128 threads handles
     int xfer_bytes_per_thread;  // dynamic shared memory per thread of variants 0..2 (0: none)

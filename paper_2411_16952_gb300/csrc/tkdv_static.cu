@@ -166,7 +166,8 @@ extern "C" int sampler_run_static(int K, const tkdv_point *point, uint64_t idx0,
         e = cudaLaunchKernel(fn, dim3(ctas), dim3(256), margs, dyn, st);
         if (e == cudaSuccess) {
             void *rargs[] = {&B, &k0, &k1};
-            e = cudaLaunchKernel(kt.refine[uni], dim3(kt.refine_smem ? sms : sms * 4), dim3(128), rargs, (size_t)kt.refine_smem, st);
+            e = cudaLaunchKernel(kt.refine[uni], dim3(sms * kt.refine_ctas), dim3(kt.refine_threads), rargs,
+                                 (size_t)kt.refine_smem, st);
         }
         if (e != cudaSuccess) return TKDV_ERR_CUDA;
     }
