@@ -39,7 +39,8 @@
 // registers (64-bit float conversions run on the FP64 pipe, 12 % busy with
 // them).  The transform's error in H3 against FP64, with that of the draw, is
 // 4.8e-7 of the root mean square (3.8e-7 with the tiles; nearly all of the
-// difference to log f/(Mg), 1.2e-5, is the draw's and unchanged).
+// difference to log f/(Mg), 1.2e-5, is the draw's and unchanged).  It serves the
+// decision; the H3 of a kept record is the double sum (fold_T, 3.8e-7).
 //
 // Rounding: the 2-norm of the 192 values is off by at most 25 roundings
 // (coefficients 1, three-level 8-point transforms 5 each, twists 3 each, the
@@ -289,6 +290,69 @@ __device__ __forceinline__ WEval warp_batch(float2 *sv, const float2 *s_tw, cons
     ev.T = fmaf(__shfl_sync(0xffffffffu, cub, 8 * ql), 1.f / (3.f * kWN), alias * (1.f / 3.f));
     ev.tail = (tails >> ql) & 1u;
     return ev;
+}
+
+// T |x|^3 of a proposal whose H3 is written out, by the double sum of Eq. (42),
+// folded: T = sum_{n=2}^{K} Re(conj(v_n) W_n), W_n = 2 sum_{k < n-k} v_k v_{n-k} +
+// [n even] v_{n/2}^2, a row n per lane, its products summed eight at a time.  Off
+// by 1.2e-7 of the root mean square of T, where the transform is off by 2.6e-7
+// (the draw adds 3.6e-7): the decision's guard covers that, the output keeps the
+// double sum.  Bound by shared-memory loads, two for a product: 1.5 ns for a kept
+// record at 128 modes (2 x 2^21 proposals, 1.16e6 accepted: 3.27 ms with a ring of
+// 16 records, 4.98 ms with all kept; 6.52 ms when the tiles served every draw).
+__device__ __forceinline__ float fold_T(const float2 *v, int K, int lane) {
+    float t = 0.f;
+#pragma unroll 1
+    for (int n = 2 + lane; n <= K; n += 32) {
+        float A = 0.f, B = 0.f;
+        int k0 = 1;
+#pragma unroll 1
+        for (; 2 * (k0 + 7) < n; k0 += 8) {
+            float a = 0.f, b = 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                const float4 p = *reinterpret_cast<const float4 *>(v + k0 - 1 + j);  // modes k0 + j, k0 + j + 1
+                const float2 q = v[n - k0 - j - 1], r = v[n - k0 - j - 2];
+                a = fmaf(p.x, q.x, a);
+                a = fmaf(-p.y, q.y, a);
+                b = fmaf(p.x, q.y, b);
+                b = fmaf(p.y, q.x, b);
+                a = fmaf(p.z, r.x, a);
+                a = fmaf(-p.w, r.y, a);
+                b = fmaf(p.z, r.y, b);
+                b = fmaf(p.w, r.x, b);
+            }
+            A += a;
+            B += b;
+        }
+        float a = 0.f, b = 0.f;
+#pragma unroll
+        for (int k = k0; k < k0 + 7; ++k) {
+            if (2 * k < n) {
+                const float2 p = v[k - 1], q = v[n - k - 1];
+                a = fmaf(p.x, q.x, a);
+                a = fmaf(-p.y, q.y, a);
+                b = fmaf(p.x, q.y, b);
+                b = fmaf(p.y, q.x, b);
+            }
+        }
+        A += a;
+        B += b;
+        A *= 2.f;
+        B *= 2.f;
+        if ((n & 1) == 0) {
+            const float2 h = v[n / 2 - 1];
+            A = fmaf(h.x, h.x, A);
+            A = fmaf(-h.y, h.y, A);
+            B = fmaf(2.f * h.x, h.y, B);
+        }
+        const float2 vn = v[n - 1];
+        t = fmaf(vn.x, A, t);
+        t = fmaf(vn.y, B, t);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
 }
 
 // Steps 5-6 for the lane's proposal (the formulas of eval_fast).
@@ -620,7 +684,7 @@ __global__ void __launch_bounds__(NT, MINB)
                     if (slot < B.ring_cap) {
                         rec = B.ring + slot * B.rec_bytes;
                         write_header(rec, ((unsigned long long)hq << 32) | lq, (uint32_t)p, 0u, sc.E0 * f.S,
-                                     sc.h3s * f.T, u0, f.delta);
+                                     sc.h3s * f.T, u0, f.delta);  // (H3 again below)
                     } else {
                         atomicAdd(&s_cnt[2], 1u);
                     }
@@ -632,6 +696,10 @@ __global__ void __launch_bounds__(NT, MINB)
                     float *xh = reinterpret_cast<float *>(
                         __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(rec), q));
                     const float sc2 = (inv * inv) * kSpecScale;
+                    if (xh) {  // the same in every lane
+                        const float T = fold_T(sv + q * kWS, sc.K, lane);
+                        if (lane == q) xh[5] = sc.h3s * (T * (rcp_rn(ev.nrm2) * f.inv));
+                    }
 #pragma unroll
                     for (int cc = 0; cc < kWK / 32; ++cc) {
                         const int m = lane + 32 * cc;
@@ -747,7 +815,6 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
             row[2] = f.d < 0.f ? 1.0 : 0.0;
             row[3] = 0.0;
             row[4] = sc.E0 * f.S;
-            row[5] = sc.h3s * f.T;
             row[6] = sc.u0s * ev.u0raw * f.inv;
             row[7] = f.S;
         }
@@ -785,6 +852,8 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
         if (!((mf >> q) & 1u)) continue;
         const float inv = __shfl_sync(0xffffffffu, f.inv, q);
         double *row = out + (b0 + q) * rowlen;
+        const float T = fold_T(sv + q * kWS, K, lane);
+        if (lane == q) row[5] = sc.h3s * (T * (rcp_rn(ev.nrm2) * f.inv));
         for (int m = lane; m < K; m += 32) {
             const float2 v = sv[q * kWS + m];
             row[8 + m] = v.x * inv;

@@ -1,0 +1,63 @@
+"""Error of H3 of the warp form's FP32 path (65..128 modes) against the oracle,
+relative to the root mean square of H3.  What is written out of a draw is off, in
+the root mean square over 8192 draws, by at most what it was when the triads of
+Eq. (42) were summed in tiles (measured on the same draws).  The H3 of the
+decision, by the transform, is seen where C3/C2 is so large that log f/(Mg) is
+nothing else: at most twice that."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def T():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2411_16952_gb300 import _build
+    _build.build()
+    import paper_2411_16952_gb300 as T
+    return T
+
+
+# K: (paper's proposal, uniform), in 1e-7
+TILED = {65: (3.826, 3.838), 96: (3.810, 3.734), 120: (3.767, 3.743), 121: (3.749, 3.730), 127: (3.841, 3.763),
+         128: (3.807, 3.740)}
+
+
+@pytest.mark.parametrize("uniform", [False, True])
+@pytest.mark.parametrize("K", sorted(TILED))
+def test_errors_are_at_most_those_of_the_tiled_sum(T, K, uniform):
+    prop, tprop = (O.UNIFORM, T.PROPOSAL_UNIFORM) if uniform else (O.PAPER, T.PROPOSAL_PAPER)
+    bp, r = 30.0, 300.0
+    pt = O.make_point(K, 1.0, bp, r, prop)
+    pt.logM = 400.0  # nothing near the threshold: every value from the FP32 path
+    S = T.Sampler(K, [T.make_point(bp, 1.0, r, tprop, logM=400.0)], sample_capacity=16)
+    idx = np.arange(8192, dtype=np.uint64)
+    g, o = S.replay(0, idx, 5), O.replay(pt, 5, 0, idx)
+    S.close()
+    fast = g["flags"] == 0
+    assert fast.sum() > 8000
+    err = np.sqrt(np.mean((g["H3"] - o["H3"])[fast] ** 2) / np.mean(o["H3"][fast] ** 2))
+    assert err <= TILED[K][uniform] * 1e-7
+
+
+@pytest.mark.parametrize("K", sorted(TILED))
+def test_h3_of_the_decision(T, K):
+    bp, r = 30.0, 1e6
+    pt = O.make_point(K, 1.0, bp, r, O.PAPER)
+    pt.logM = 0.0
+    S = T.Sampler(K, [T.make_point(bp, 1.0, r, T.PROPOSAL_PAPER, logM=0.0)], sample_capacity=16)
+    idx = np.arange(8192, dtype=np.uint64)
+    g, o = S.replay(0, idx, 5), O.replay(pt, 5, 0, idx)
+    S.close()
+    fast = g["flags"] == 0
+    assert fast.sum() > 8000
+    h3 = bp * r / (K * K) * o["H3"][fast]
+    err = math.sqrt(np.mean((g["delta"] - o["delta"])[fast] ** 2) / np.mean(h3**2))
+    assert err <= 2 * TILED[K][0] * 1e-7
