@@ -40,7 +40,7 @@
 // them).  The transform's error in H3 against FP64, with that of the draw, is
 // 4.8e-7 of the root mean square (3.8e-7 with the tiles; nearly all of the
 // difference to log f/(Mg), 1.2e-5, is the draw's and unchanged).  It serves the
-// decision; the H3 of a kept record is the double sum (fold_T, 3.8e-7).
+// decision; H3 and log f/(Mg) of a kept record have the double sum (fold_T, 3.8e-7).
 //
 // Rounding: the 2-norm of the 192 values is off by at most 25 roundings
 // (coefficients 1, three-level 8-point transforms 5 each, twists 3 each, the
@@ -292,14 +292,14 @@ __device__ __forceinline__ WEval warp_batch(float2 *sv, const float2 *s_tw, cons
     return ev;
 }
 
-// T |x|^3 of a proposal whose H3 is written out, by the double sum of Eq. (42),
+// T |x|^3 of a proposal whose H3 and log f/(Mg) are written out, by the double sum of Eq. (42),
 // folded: T = sum_{n=2}^{K} Re(conj(v_n) W_n), W_n = 2 sum_{k < n-k} v_k v_{n-k} +
 // [n even] v_{n/2}^2, a row n per lane, its products summed eight at a time.  Off
 // by 1.2e-7 of the root mean square of T, where the transform is off by 2.6e-7
 // (the draw adds 3.6e-7): the decision's guard covers that, the output keeps the
 // double sum.  Bound by shared-memory loads, two for a product: 1.5 ns for a kept
 // record at 128 modes (2 x 2^21 proposals, 1.16e6 accepted: 3.27 ms with a ring of
-// 16 records, 4.98 ms with all kept; 6.52 ms when the tiles served every draw).
+// 16 records, 5.00 ms with all kept; 6.52 ms when the tiles served every draw).
 __device__ __forceinline__ float fold_T(const float2 *v, int K, int lane) {
     float t = 0.f;
 #pragma unroll 1
@@ -684,7 +684,7 @@ __global__ void __launch_bounds__(NT, MINB)
                     if (slot < B.ring_cap) {
                         rec = B.ring + slot * B.rec_bytes;
                         write_header(rec, ((unsigned long long)hq << 32) | lq, (uint32_t)p, 0u, sc.E0 * f.S,
-                                     sc.h3s * f.T, u0, f.delta);  // (H3 again below)
+                                     sc.h3s * f.T, u0, f.delta);  // (H3 and log f/(Mg) again below)
                     } else {
                         atomicAdd(&s_cnt[2], 1u);
                     }
@@ -697,8 +697,13 @@ __global__ void __launch_bounds__(NT, MINB)
                         __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(rec), q));
                     const float sc2 = (inv * inv) * kSpecScale;
                     if (xh) {  // the same in every lane
-                        const float T = fold_T(sv + q * kWS, sc.K, lane);
-                        if (lane == q) xh[5] = sc.h3s * (T * (rcp_rn(ev.nrm2) * f.inv));
+                        WEval out = ev;
+                        out.T = fold_T(sv + q * kWS, sc.K, lane);
+                        if (lane == q) {
+                            const Fast g = warp_eval<UNIF>(out, sc, wa);
+                            xh[5] = sc.h3s * g.T;
+                            xh[7] = g.delta;
+                        }
                     }
 #pragma unroll
                     for (int cc = 0; cc < kWK / 32; ++cc) {
@@ -807,14 +812,24 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
     const bool valid = lane < kWQ && ((vmask >> lane) & 1u);
     const bool slow = fabsf(f.d) < f.guard || ev.tail || wa < kTailBucket;
     const size_t rowlen = 8 + 2 * (size_t)K;
+    // the outputs of the proposals decided in FP32, T by the double sum
+    const unsigned mf = __ballot_sync(0xffffffffu, valid && !slow);
+    WEval eo = ev;
+    for (int q = 0; q < kWQ; ++q) {
+        if (!((mf >> q) & 1u)) continue;
+        const float T = fold_T(sv + q * kWS, K, lane);
+        if (lane == q) eo.T = T;
+    }
     if (valid && !slow) {
+        const Fast g = warp_eval<UNIF>(eo, sc, wa);
         double *row = out + (b0 + lane) * rowlen;
         {
-            row[0] = f.delta;
+            row[0] = g.delta;
             row[1] = f.lnU;
             row[2] = f.d < 0.f ? 1.0 : 0.0;
             row[3] = 0.0;
             row[4] = sc.E0 * f.S;
+            row[5] = sc.h3s * g.T;
             row[6] = sc.u0s * ev.u0raw * f.inv;
             row[7] = f.S;
         }
@@ -847,13 +862,10 @@ __global__ void __launch_bounds__(32 * kReplayWarps) k_replay_warp(const PointCo
         }
     }
     // projected state of the proposals decided in FP32, written by the warp
-    const unsigned mf = __ballot_sync(0xffffffffu, valid && !slow);
     for (int q = 0; q < kWQ; ++q) {
         if (!((mf >> q) & 1u)) continue;
         const float inv = __shfl_sync(0xffffffffu, f.inv, q);
         double *row = out + (b0 + q) * rowlen;
-        const float T = fold_T(sv + q * kWS, K, lane);
-        if (lane == q) row[5] = sc.h3s * (T * (rcp_rn(ev.nrm2) * f.inv));
         for (int m = lane; m < K; m += 32) {
             const float2 v = sv[q * kWS + m];
             row[8 + m] = v.x * inv;
