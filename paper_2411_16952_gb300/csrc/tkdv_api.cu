@@ -562,6 +562,31 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
         h->err = rce ? msg : std::string("no CUDA device: ") + cudaGetErrorString(e);
         return bail(rce ? rce : TKDV_ERR_CUDA);
     }
+    auto alloc = [&](void **p, size_t bytes) -> int {
+        cudaError_t ee = cudaMalloc(p, bytes ? bytes : 16);
+        if (ee != cudaSuccess) {
+            h->err = std::string("cudaMalloc: ") + cudaGetErrorString(ee);
+            return ee == cudaErrorMemoryAllocation ? TKDV_ERR_OOM : TKDV_ERR_CUDA;
+        }
+        return TKDV_OK;
+    };
+    int rc;
+    // the envelopes first, in the FP64 queue, which is free before the first
+    // run: a point whose search fails answers so whatever else is wrong
+    {
+        const int rca = alloc(&h->d_refine, sizeof(RefineItem) * (size_t)kRefineCap);
+        const std::string why = h->err;
+        std::string msg;
+        rc = find_envelopes(h, h->d_refine, msg);
+        if (!rc && rca) {
+            rc = rca;
+            h->err = why;
+        }
+        if (rc) {
+            if (!msg.empty()) h->err = msg;
+            return bail(rc);
+        }
+    }
     for (int u = 0; u < 2 && h->kt.refine_smem && e == cudaSuccess; ++u)
         e = cudaFuncSetAttribute(h->kt.refine[u], cudaFuncAttributeMaxDynamicSharedMemorySize, h->kt.refine_smem);
     if (e != cudaSuccess) {
@@ -655,15 +680,6 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
     }
     h->rec_bytes = record_bytes(h->K);
     const unsigned long long cap = opt->sample_capacity;
-    auto alloc = [&](void **p, size_t bytes) -> int {
-        cudaError_t ee = cudaMalloc(p, bytes ? bytes : 16);
-        if (ee != cudaSuccess) {
-            h->err = std::string("cudaMalloc: ") + cudaGetErrorString(ee);
-            return ee == cudaErrorMemoryAllocation ? TKDV_ERR_OOM : TKDV_ERR_CUDA;
-        }
-        return TKDV_OK;
-    };
-    int rc;
     if ((rc = alloc(&h->d_pts, sizeof(PointConst) * n_points))) return bail(rc);
     if ((rc = alloc(&h->d_stats, state_bytes(h)))) return bail(rc);
     {
@@ -673,7 +689,6 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
         h->d_counters = t->counters;
     }
     if ((rc = alloc(&h->d_ring, h->rec_bytes * cap))) return bail(rc);
-    if ((rc = alloc(&h->d_refine, sizeof(RefineItem) * (size_t)kRefineCap))) return bail(rc);
     if (opt->cuda_stream) {
         h->stream = (cudaStream_t)opt->cuda_stream;
     } else {
@@ -683,13 +698,6 @@ int sampler_create_ex(const tkdv_point *points, int n_points, const tkdv_options
             return bail(TKDV_ERR_CUDA);
         }
         h->own_stream = true;
-    }
-    {
-        std::string msg;
-        if ((rc = find_envelopes(h, h->d_refine, msg))) {  // the queue is free before the first run
-            if (!msg.empty()) h->err = msg;
-            return bail(rc);
-        }
     }
     for (int p = 0; p < n_points; ++p) {
         fill_point_const(h->K, h->pts[p], h->sigma2[p].data(), h->logM[p], false, h->pc_triad[p]);
