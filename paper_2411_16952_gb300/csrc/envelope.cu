@@ -376,8 +376,8 @@ cudaError_t launch(const EnvPoint *pts, int P, int K, unsigned long long *best, 
     const size_t smem = sizeof(double) * kEnvWarps * 32 * VPL * (1 + 2 * kHist);
     cudaError_t e = cudaFuncSetAttribute(k_envelope<VPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_envelope<VPL><<<(tasks + kEnvWarps - 1) / kEnvWarps, 32 * kEnvWarps, smem, st>>>(pts, P, K, K + 13, best);
-    return cudaGetLastError();
+    return launch_kernel(k_envelope<VPL>, (tasks + kEnvWarps - 1) / kEnvWarps, 32 * kEnvWarps, smem, st, pts, P, K, K + 13,
+                         best);
 }
 
 }  // namespace

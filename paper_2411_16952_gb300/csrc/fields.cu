@@ -75,8 +75,8 @@ cudaError_t launch_field_max(const unsigned char *ring, unsigned long long rec_b
                              const PointConst *pts, float *umax, int *jmax, cudaStream_t st) {
     if (!n) return cudaSuccess;
     const unsigned long long blocks = std::min<unsigned long long>((n + 3) / 4, 65535ull * 16);
-    k_field_max<<<(unsigned)blocks, 128, 0, st>>>(ring, rec_bytes, n, K, pts, nullptr, nullptr, umax, jmax, nullptr);
-    return cudaGetLastError();
+    return launch_kernel(k_field_max, (unsigned)blocks, 128, 0, st, ring, rec_bytes, n, K, pts, nullptr, nullptr, umax, jmax,
+                         nullptr);
 }
 
 // ---- the 1-in-m event ----------------------------------------------------------
@@ -226,17 +226,19 @@ cudaError_t launch_extreme(const unsigned char *ring, unsigned long long rec_byt
     int *jmax = (int *)(umax + m);
     *out = ExtremeBufs{&s->n_match, list, idx, umax, jmax};
     const unsigned blocks = (unsigned)std::min<unsigned long long>((n + 1023) / 1024, 608);
-    k_sel_init<<<1, 256, 0, st>>>(s, m);
-    k_sel_gather<<<blocks, 256, 0, st>>>(ring, rec_bytes, n, point, s, key, pos);
-    for (int d = 5; d >= 0; --d) k_sel_pass<false><<<blocks, 256, 0, st>>>(s, key, pos, d * kDigit, d == 5, d == 0);
+    cudaError_t e = launch_kernel(k_sel_init, 1, 256, 0, st, s, m);
+    if (e == cudaSuccess) e = launch_kernel(k_sel_gather, blocks, 256, 0, st, ring, rec_bytes, n, point, s, key, pos);
+    for (int d = 5; d >= 0 && e == cudaSuccess; --d)
+        e = launch_kernel(k_sel_pass<false>, blocks, 256, 0, st, s, key, pos, d * kDigit, d == 5, d == 0);
     int digits = 1;
     while ((n - 1) >> (digits * kDigit)) ++digits;
-    for (int d = digits - 1; d >= 0; --d)
-        k_sel_pass<true><<<blocks, 256, 0, st>>>(s, key, pos, d * kDigit, d == digits - 1, d == 0);
-    k_sel_list<<<blocks, 256, 0, st>>>(s, key, pos, list, m);
+    for (int d = digits - 1; d >= 0 && e == cudaSuccess; --d)
+        e = launch_kernel(k_sel_pass<true>, blocks, 256, 0, st, s, key, pos, d * kDigit, d == digits - 1, d == 0);
+    if (e == cudaSuccess) e = launch_kernel(k_sel_list, blocks, 256, 0, st, s, key, pos, list, m);
     const unsigned fb = (unsigned)std::min<unsigned long long>((m + 3) / 4, 65535ull * 16);
-    k_field_max<<<fb, 128, 0, st>>>(ring, rec_bytes, m, K, pts, list, &s->n_list, umax, jmax, idx);
-    return cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_kernel(k_field_max, fb, 128, 0, st, ring, rec_bytes, m, K, pts, list, &s->n_list, umax, jmax, idx);
+    return e;
 }
 
 }  // namespace tkdv

@@ -199,6 +199,19 @@ inline size_t record_bytes(int K) {
     return (b + 15) & ~(size_t)15;
 }
 
+// Launch of a kernel that returns this launch's own error.  (cudaGetLastError
+// behind a launch also returns, and so lets it fail for, what an earlier call of
+// the thread left there, an allocation that did not fit for instance.)
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*fn)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    return cudaLaunchKernelEx(&c, fn, static_cast<P>(args)...);
+}
+
 // One point of the envelope search on the device (envelope.cu): log f/g =
 // cS S + cH T + cQ ln Q over real amplitudes, cH >= 0 (see there).
 struct EnvPoint {
