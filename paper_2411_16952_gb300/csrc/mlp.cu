@@ -694,7 +694,8 @@ int tkdv_mlp_step(tkdv_mlp *m, float lr, float tau, int update, double *loss, fl
     if (!m->d_done) return mfail(m, TKDV_ERR_INVALID_ARG, "the training set was refused");  // (allocated last)
     const int P = m->P;
     const __nv_bfloat16 *wb = m->d_wb[m->cur];
-    k_forward<<<P, 64>>>(wb, m->d_feats, m->d_h1, m->d_h2, m->d_out, m->d_K, m->d_wpaper, m->d_wprime, m->d_slw);
+    MCK(launch_kernel(k_forward, P, 64, 0, 0, wb, m->d_feats, m->d_h1, m->d_h2, m->d_out, m->d_K, m->d_wpaper, m->d_wprime,
+                      m->d_slw));
     {
         const float *s = m->d_s, *z = m->d_z, *wpr = m->d_wprime, *slw = m->d_slw;
         const unsigned long long *r0 = m->d_row0, *nr = m->d_nrows;
@@ -708,15 +709,16 @@ int tkdv_mlp_step(tkdv_mlp *m, float lr, float tau, int update, double *loss, fl
     float c1 = 1.f, c2 = 1.f;
     const float b1 = 0.9f, b2 = 0.999f;
     if (update) {
-        m->step += 1;
-        c1 = 1.f - std::pow(b1, (float)m->step);
-        c2 = 1.f - std::pow(b2, (float)m->step);
+        c1 = 1.f - std::pow(b1, (float)(m->step + 1));
+        c2 = 1.f - std::pow(b2, (float)(m->step + 1));
     }
-    k_backward<<<(NPARAM + 255) / 256, 256, sizeof(float) * 2 * P * H>>>(
-        wb, m->d_feats, m->d_h1, m->d_h2, m->d_dout, P, m->d_grad, update ? 1 : 0, m->d_master, m->d_m1, m->d_m2,
-        m->d_wb[m->cur ^ 1], lr, b1, b2, 1e-8f, c1, c2);
-    MCK(cudaGetLastError());
-    if (update) m->cur ^= 1;
+    MCK(launch_kernel(k_backward, (NPARAM + 255) / 256, 256, sizeof(float) * 2 * P * H, 0, wb, m->d_feats, m->d_h1, m->d_h2,
+                      m->d_dout, P, m->d_grad, update ? 1 : 0, m->d_master, m->d_m1, m->d_m2, m->d_wb[m->cur ^ 1], lr, b1,
+                      b2, 1e-8f, c1, c2));
+    if (update) {  // the masters, their copies and the step count go together
+        m->step += 1;
+        m->cur ^= 1;
+    }
     // losses and gradient in one copy
     if (loss || grad_out)
         MCK(cudaMemcpyAsync(m->h_lg, m->d_loss, 4 * (size_t)(grad_out ? TKDV_MAX_POINTS + NPARAM : P),

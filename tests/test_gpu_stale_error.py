@@ -36,3 +36,23 @@ def test_calls_after_a_failed_allocation(T):
     st = T.sampler_batch_run([T.make_point(2.0, 1.0, 1.0)], T.make_options(8, sample_capacity=16), [1 << 14], 3)
     assert st[0]["n_accepted"] == S.stats()[0]["n_accepted"] == len(umax)
     S.close()
+
+
+def test_training_step_after_a_failed_allocation(T):
+    K, n, rng = 8, 512, np.random.default_rng(1)
+    s = rng.random((n, K)).astype(np.float32)
+    s /= s.sum(1, keepdims=True)
+    w0 = (0.1 * rng.standard_normal(T.MLP_NPARAM)).astype(np.float32)
+    got = []
+    for fail in (False, True):
+        m = T.tkdv_mlp_create(0)
+        T.tkdv_mlp_set_params(m, w0)
+        T.tkdv_mlp_set_data(m, [K], [T.tkdv_mlp_features(K, 2.0, 1.0, 1.0)], [np.ones(K)], [s])
+        for _ in range(3):
+            if fail:
+                _fail(T)
+            loss, grad = T.tkdv_mlp_step(m, lr=1e-2, tau=1.0, update=True, want_grad=True)
+        got.append([np.array(loss), grad, *T.tkdv_mlp_get_params(m)])
+        T.tkdv_mlp_destroy(m)
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
