@@ -1170,8 +1170,9 @@ __device__ __forceinline__ double seg_sum(double v) {
 // draws finish: consecutive draws together, as in this form.
 template <int KMAX, bool UNIF>
 __device__ __noinline__ void refine_serial(const DevBufs &B, uint32_t n, uint32_t k0, uint32_t k1) {
-    // a short queue goes to the first warps of all CTAs, not to all warps of the first
-    for (uint32_t i = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31); i < n;
+    // a short queue goes to the first four warps of the CTAs, one per scheduler,
+    // and not to all warps of a few
+    for (uint32_t i = ((threadIdx.x >> 7) * gridDim.x + blockIdx.x) * 128 + (threadIdx.x & 127); i < n;
          i += gridDim.x * blockDim.x) {
         const RefineItem it = B.refine[i];
         const PointConst *P = B.pts + it.point;
