@@ -122,7 +122,8 @@ typedef struct {
     int h3_mode;              /* TKDV_H3_* */
     int grid_N;               /* grid points of the grid form (TKDV_H3_GRID_BF16X3, or TKDV_H3_AUTO with
                                  K <= 64): multiple of 32, > 3K, <= 256; 0: the smallest such (128 for K = 32) */
-    uint64_t sample_capacity; /* accepted records kept per handle (ring; excess is counted, not kept) */
+    uint64_t sample_capacity; /* accepted records kept per handle (ring; excess is counted, not kept; which
+                                 records, and so the points' n_dropped, is then unspecified) */
     void *cuda_stream;        /* cudaStream_t to launch on; NULL: the handle makes its own */
     int use_graph;            /* 1: launch each run as one CUDA graph (default), 0: plain launches */
     int ctas_per_sm;          /* 0: occupancy maximum; else persistent CTAs per SM */
@@ -229,7 +230,9 @@ int sampler_stats(tkdv_sampler *h, tkdv_stats *out, int n_out);
 
 /* sampler_samples: waits, then copies up to max_records accepted records
    (tkdv_record_bytes(K) bytes each, unordered) to dst, a host buffer if
-   dst_on_device == 0, else a device buffer; *n_out = records copied. */
+   dst_on_device == 0, else a device buffer; *n_out = records copied.  A copy
+   to a device buffer runs on the legacy default stream and may still be on its
+   way at return; the handle's next runs wait for it. */
 int sampler_samples(tkdv_sampler *h, void *dst, int dst_on_device, uint64_t max_records,
                     uint64_t *n_out);
 

@@ -295,12 +295,17 @@ int build_args(tkdv_sampler *h, const unsigned long long *idx0, const unsigned l
     // Chunks: a whole number m of them per persistent worker (a CTA of the
     // triad form, a warpgroup of the grid form), between 1 and 64 proposals per
     // thread, so that the last round is full: 8, or more where 64 proposals
-    // per thread are not enough; in the triad form, whose CTAs do not share an
-    // SM's issue slots as warpgroups do, 32 or 16 where a chunk still has 16
-    // trips of the CTA's loop.  With the largest chunks whatever the count,
+    // per thread are not enough.  With the largest chunks whatever the count,
     // 2^25 proposals at 64 modes were 13.5 rounds that took 14 (6.22 -> 6.12
-    // ms), 8 x 2^22 in the triad form 6.7 that took 7 (3.43 -> 3.37 ms), 2 x
-    // 2^21 at 128 modes 7.7 that took 8 (3.41 -> 3.31 ms).
+    // ms), 8 x 2^22 in the triad form 6.7 that took 7 (3.43 -> 3.34 ms), 2 x
+    // 2^21 at 128 modes 7.7 that took 8 (3.41 -> 3.31 ms).  In the triad form 16
+    // or 32 where a chunk still has 16 trips of the CTA's loop (us with m = 8, 16,
+    // 32; trips of a CTA in the whole run): 8 x 2^22 at 32 modes 3,298, 3,271, 3,232
+    // and again 3,313, 3,241, 3,248 (431), 8 x 2^23 6,447, 6,504, 6,423 (862), 2^25
+    // at 16 modes 1,566, 1,500, 1,539 (431), 2^26 2,945, 2,995, 2,988 (862): within
+    // 1.5 % of the best of the three.  With fewer trips the ends of the chunks
+    // count: 2^20 at 16 modes 85, 94, 96 (13), 2^23 419, 423, 442 (108), 2^24 at 8
+    // modes 1,279, 1,309, 1,359 (216), 4 x 2^21 at 40 modes 2,507, 2,513, 2,471 (216).
     const bool grid = is_grid(h), warp = h->kmax == 128;
     const unsigned long long thr = grid ? 128ull : (unsigned long long)h->launch.threads;
     const unsigned long long trip = warp ? 32ull : thr;  // (the warp form: four proposals per warp)
